@@ -41,7 +41,7 @@ struct irtps_batch {
   uint32_t *iter_dev = nullptr;
   // launch geometry
   int pyr_levels = 0;
-  std::vector<int> pyr_blocks;
+  int pyr_blocks = 0;
   int hz_blocks = 0;  // batched horizon launch (early escape)
   int ps_blocks = 0, cg_blocks = 0;
   unsigned n_items = 0;
@@ -210,7 +210,7 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
 
 int enqueue_trace(irtps_batch &b, uint32_t iter, bool captured, bool timed) {
   BSTAGE(ST_TRACE, true);
-  BCK(irtps::build_pyramid_batch(b.stream, b.d_pyr, b.n, b.pyr_levels, b.pyr_blocks.data()), "pyramid launch");
+  BCK(irtps::build_pyramid_batch(b.stream, b.d_pyr, b.n, b.pyr_levels, b.pyr_blocks), "pyramid launch");
   BCK(irtps::launch_horizon_batch(b.stream, b.d_pyr, b.n, b.hz_blocks), "horizon bounds");
   if (b.shared) BCK(irtps::launch_parts_batch(b.stream, true, b.d_reduce, b.n, b.reduce_blocks), "partial sums");
   BCK(irtps::launch_trace_batch(b.stream, b.C, b.shared, b.d_trace, b.n, b.n_items, b.d_stats[b.n].counts,
@@ -420,7 +420,7 @@ int irtps_batch_create(irtps_batch **out, irtps_ctx *const *objs, int n_obj, int
     return bail(IRTPS_ECUDA);
   b.stream = b.own_stream;
 
-  // pyramid: per level, each object's block range (none beyond its levels)
+  // pyramid: each object's range of tiles
   std::vector<irtps::PyrObj> pyr(n_obj);
   for (int i = 0; i < n_obj; ++i) {
     irtps::fill_pyr_obj(objs[i]->c, pyr[i]);
@@ -431,13 +431,10 @@ int irtps_batch_create(irtps_batch **out, irtps_ctx *const *objs, int n_obj, int
     pyr[i].hz_blk = b.hz_blocks;
     if (pyr[i].hz) b.hz_blocks += (objs[i]->c.H * objs[i]->c.W + 127) / 128;
   }
-  b.pyr_blocks.assign(b.pyr_levels, 0);
-  for (int l = 0; l < b.pyr_levels; ++l)
-    for (int i = 0; i < n_obj; ++i) {
-      pyr[i].blk[l] = b.pyr_blocks[l];
-      if (l < pyr[i].levels)
-        b.pyr_blocks[l] += (pyr[i].lw[l] * pyr[i].lh[l] + irtps::kPyrThreads - 1) / irtps::kPyrThreads;
-    }
+  for (int i = 0; i < n_obj; ++i) {
+    pyr[i].blk = b.pyr_blocks;
+    b.pyr_blocks += irtps::pyramid_tiles(objs[i]->c.H, objs[i]->c.W);
+  }
   // PS: ceil(P / 256) blocks per object
   const size_t ps_bytes = irtps::ps_args_bytes();
   std::vector<unsigned char> ps(ps_bytes * n_obj), ps0(ps_bytes * n_obj);
@@ -553,7 +550,7 @@ int irtps_batch_iterate(irtps_batch *x, int n_iter, const int *spp, const int *b
   {  // kernels per iteration: pyramid levels, trace, PS, the solve's, two of D_H (+ counter)
     int k = 1 + 1 + solve_kernels(b) + 2 + (b.use_graph ? 1 : 0) + (b.shared ? 2 : 0) + (b.hz_blocks > 0 ? 1 : 0) +
             irls_kernels(b);
-    for (int l = 0; l < b.pyr_levels; ++l) k += b.pyr_blocks[l] > 0 ? 1 : 0;
+    k += b.pyr_levels > irtps::kPyrTileLevels ? 2 : 1;
     b.stats.launches += (unsigned long long)k * n_iter;
   }
   for (irtps_ctx *o : b.objs) o->c.t += (uint32_t)n_iter;

@@ -43,7 +43,7 @@ int dalloc(Ctx &c, T **p, size_t n, const char *what) {
 }
 
 void release(Ctx &c) {
-  void *bufs[] = {c.env, c.d_lights, c.horizon, c.shared_part, c.images, c.lbar, c.depth, c.depth_prev, c.nrm, c.albedo, c.valid, c.pmin, c.pmax,
+  void *bufs[] = {c.env, c.d_lights, c.horizon, c.shared_part, c.images, c.lbar, c.depth, c.depth_prev, c.nrm, c.albedo, c.valid, c.pmax, c.planes,
                   c.cg_x, c.cg_b, c.cg_r, c.cg_z, c.cg_p, c.cg_ap, c.part, c.dstats, c.next_item, c.cg_ctl,
                   c.mg_x0, c.mg_x1, c.mg_b, c.mg_wh, c.mg_wv, c.mg_wh_unit, c.mg_wv_unit, c.iter_dev, c.holes,
                   c.fill_v, c.fill_w, c.sp_ch, c.sp_cw, c.sp_mu, c.sp_nu, c.sp_t, c.ps_pix, c.ps_mask,
@@ -412,7 +412,7 @@ int irtps_create(irtps_ctx **out, int H, int W, int K, int C, const float *light
       (rc = dalloc(c, &c.ps_pix, P, "masked-pixel list")) || (rc = dalloc(c, &c.ps_mask, P, "masked-pixel list")) ||
       (rc = dalloc(c, &c.ps_rhs, (size_t)9 * P, "masked-pixel list")) ||
       (rc = dalloc(c, &c.ps_count, 1, "masked-pixel list")) ||
-      (rc = dalloc(c, &c.pmin, (size_t)total, "pyramid")) || (rc = dalloc(c, &c.pmax, (size_t)total, "pyramid")) ||
+      (rc = dalloc(c, &c.pmax, (size_t)total, "pyramid")) || (rc = dalloc(c, &c.planes, (size_t)total, "pyramid")) ||
       (rc = dalloc(c, &c.cg_x, P, "cg")) || (rc = dalloc(c, &c.cg_b, P, "cg")) ||
       (rc = dalloc(c, &c.cg_r, P, "cg")) || (rc = dalloc(c, &c.cg_z, P, "cg")) ||
       (rc = dalloc(c, &c.cg_p, 2 * P, "cg")) || (rc = dalloc(c, &c.cg_ap, 2 * P, "cg")) ||

@@ -122,7 +122,8 @@ struct Ctx {
   unsigned long long *ps_mask = nullptr;  // right-hand sides (9 floats each), count
   float *ps_rhs = nullptr;
   unsigned *ps_count = nullptr;
-  float *pmin = nullptr, *pmax = nullptr;  // pyramid, all levels
+  float *pmax = nullptr;          // pyramid of maxima, all levels
+  uint2 *planes = nullptr;        // bounding planes of the same nodes
   int levels = 0;
   int trace_blocks = 0;           // resident blocks of the persistent trace grid (0: one lane per item)
   int mip_cut = 0;                // top pyramid levels the march leaves out (tuning; results do not change)
@@ -158,6 +159,7 @@ struct Ctx {
     Field f;
     f.depth = depth;
     f.pmax = pmax;
+    f.planes = planes;
     f.H = H;
     f.W = W;
     f.Wc = W - 1;
@@ -185,15 +187,17 @@ namespace irtps {
 // Pyramid of one object in a batched build.
 struct PyrObj {
   const float *depth;
-  float *prev;  // when set, level 0 also copies depth here (D_H reference)
-  float *pmin, *pmax;
+  float *prev;  // when set, the build also copies depth here (D_H reference)
+  float *pmax;
+  uint2 *planes;
   int H, W, levels;
   int off[kMaxLevels], lw[kMaxLevels], lh[kMaxLevels];
-  int blk[kMaxLevels];  // first block of the object in the launch of each level
+  int blk;              // first block of the object in the tile launch
   float *hz;            // horizon bounds (null: none)
   int hz_blk;           // first block of the object in the batched horizon launch
 };
 constexpr int kPyrThreads = 256;
+constexpr int kPyrTile = 32, kPyrTileLevels = 6;  // cells a side of a tile; levels it builds (32 cells = a node of level 5)
 
 // trace.cu
 cudaError_t build_pyramid(Ctx &c);
@@ -216,7 +220,8 @@ inline bool early_escape_on(const Ctx &c, int spp, bool batched = false) {
 }
 cudaError_t launch_horizon(Ctx &c, int spp);  // horizon bounds of the current surface (after the pyramid)
 void fill_pyr_obj(const Ctx &c, PyrObj &o);
-cudaError_t build_pyramid_batch(cudaStream_t s, const PyrObj *d_objs, int n, int levels, const int *blocks);
+cudaError_t build_pyramid_batch(cudaStream_t s, const PyrObj *d_objs, int n, int levels, int blocks);
+int pyramid_tiles(int H, int W);  // blocks of one object in the tile launch
 cudaError_t launch_horizon_batch(cudaStream_t s, const PyrObj *d_objs, int n, int blocks);
 cudaError_t launch_trace(Ctx &c, const int32_t *pixels, int n_pix, int spp, int bounces, uint64_t seed,
                          uint32_t iter, uint32_t stream, float *out, int32_t *rec, bool iter_from_device = false,

@@ -12,84 +12,181 @@
 namespace irtps {
 
 // ---------------------------------------------------------------------------
-// Min / max pyramid.  Level 0: one node per cell, over its 4 vertex heights.
-// Level l: one node per 2x2 block of level l-1 nodes (clipped at the border).
+// Pyramids of the surface.  Level 0: one node per cell, over its 4 vertex heights;
+// level l: one node per 2x2 block of level l-1 nodes (clipped at the border).  Every node
+// keeps its maximum (horizon bounds, surface maximum) and an upper bounding plane
+// (the march, see plane_pack in geom.cuh): at level 0 the mean slopes of the cell and the
+// least offset over its vertices, above it the mean slopes of the children and the least
+// offset over the corners of the children's planes (3 % more node visits than offsets over all
+// vertices), or a flat plane at the maximum where that lies lower at the node's centre.  All roundings go up.
+//
+// Two launches build all levels: blocks of 32 x 32 cells carry levels 0 to 5 in shared
+// memory, then one block per object the few nodes above them.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void pyramid_leaf_node(const float *__restrict__ depth, int W, int Wc, int i,
-                                                  float *__restrict__ pmin, float *__restrict__ pmax) {
-  const int cy = i / Wc, cx = i - cy * Wc;
+struct PyrNode {
+  float mx, gx, gy, c;  // maximum; plane without its slack
+};
+
+__device__ __forceinline__ PyrNode pyramid_leaf_node(const float *__restrict__ depth, int W, int cy, int cx) {
   const float *r = depth + (size_t)cy * W + cx;
-  const float a = r[0], b = r[1], c = r[W], d = r[W + 1];
-  pmin[i] = fminf(fminf(a, b), fminf(c, d));
-  pmax[i] = fmaxf(fmaxf(a, b), fmaxf(c, d));
+  const float h00 = r[0], h01 = r[1], h10 = r[W], h11 = r[W + 1];
+  PyrNode n;
+  n.mx = fmaxf(fmaxf(h00, h01), fmaxf(h10, h11));
+  n.gx = bf16_round(0.5f * ((h01 - h00) + (h11 - h10)));
+  n.gy = bf16_round(0.5f * ((h10 - h00) + (h11 - h01)));
+  if (!(fabsf(n.gx) + fabsf(n.gy) < 1e30f)) n.gx = n.gy = 0.0f;
+  const float x0 = (float)cx, x1 = (float)(cx + 1), y0 = (float)cy, y1 = (float)(cy + 1);
+  n.c = fmaxf(fmaxf(__fmaf_ru(-n.gx, x0, __fmaf_ru(-n.gy, y0, h00)), __fmaf_ru(-n.gx, x1, __fmaf_ru(-n.gy, y0, h01))),
+              fmaxf(__fmaf_ru(-n.gx, x0, __fmaf_ru(-n.gy, y1, h10)), __fmaf_ru(-n.gx, x1, __fmaf_ru(-n.gy, y1, h11))));
+  return n;
 }
 
-__device__ __forceinline__ void pyramid_up_node(const float *__restrict__ cmin, const float *__restrict__ cmax,
-                                                int cw, int ch, int w, int i, float *__restrict__ pmin,
-                                                float *__restrict__ pmax) {
-  const int y = i / w, x = i - y * w;
-  float lo = __int_as_float(0x7f800000), hi = -lo;
-  for (int dy = 0; dy < 2; ++dy) {
-    const int yy = 2 * y + dy;
-    if (yy >= ch) break;
-    for (int dx = 0; dx < 2; ++dx) {
-      const int xx = 2 * x + dx;
-      if (xx >= cw) break;
-      lo = fminf(lo, cmin[yy * cw + xx]);
-      hi = fmaxf(hi, cmax[yy * cw + xx]);
+// Node (y, x) of level l from its children child(dy, dx), nodes (2y + dy, 2x + dx) of a cw x ch level.
+template <typename F>
+__device__ __forceinline__ PyrNode pyramid_up_node(F &&child, int cw, int ch, int l, int y, int x, int Wc, int Hc) {
+  PyrNode k[4], n;
+  bool in[4];
+  n.mx = __int_as_float(0xff800000);
+  float sx = 0.0f, sy = 0.0f, cnt = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    in[i] = 2 * y + (i >> 1) < ch && 2 * x + (i & 1) < cw;
+    if (!in[i]) continue;
+    k[i] = child(i >> 1, i & 1);
+    n.mx = fmaxf(n.mx, k[i].mx);
+    sx += k[i].gx;
+    sy += k[i].gy;
+    cnt += 1.0f;
+  }
+  n.gx = bf16_round(sx / cnt);
+  n.gy = bf16_round(sy / cnt);
+  n.c = __int_as_float(0xff800000);
+  const int half = 1 << (l - 1);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (!in[i]) continue;
+    const int X0 = (2 * x + (i & 1)) * half, Y0 = (2 * y + (i >> 1)) * half;
+    const float x0 = (float)X0, x1 = (float)min(X0 + half, Wc), y0 = (float)Y0, y1 = (float)min(Y0 + half, Hc);
+    const float dx = __fsub_ru(k[i].gx, n.gx), dy = __fsub_ru(k[i].gy, n.gy);
+    const float ex = fmaxf(__fmul_ru(dx, x0), __fmul_ru(dx, x1)), ey = fmaxf(__fmul_ru(dy, y0), __fmul_ru(dy, y1));
+    n.c = fmaxf(n.c, __fadd_ru(k[i].c, __fadd_ru(ex, ey)));
+  }
+  const float xm = (float)((2 * x + 1) * half), ym = (float)((2 * y + 1) * half);
+  if (!(fmaf(n.gx, xm, fmaf(n.gy, ym, n.c)) <= n.mx)) {
+    n.gx = n.gy = 0.0f;
+    n.c = n.mx;
+  }
+  return n;
+}
+
+__device__ __forceinline__ void pyramid_store(const PyrObj &o, int l, int y, int x, const PyrNode &n) {
+  const int i = o.off[l] + y * o.lw[l] + x;
+  o.pmax[i] = n.mx;
+  o.planes[i] = plane_pack(n.gx, n.gy, __fadd_ru(n.c, plane_slack(n.gx, n.gy, (float)o.W, (float)o.H)));
+}
+
+// Levels 0 .. 5 of one 32 x 32 tile of cells (256 threads).
+__device__ __forceinline__ void pyramid_tile(const PyrObj &o, int tile) {
+  __shared__ PyrNode s_n[2][kPyrTile * kPyrTile / 4];  // two levels in turn (level 0 stays in registers)
+  const int W = o.W, Wc = W - 1, Hc = o.H - 1;
+  const int tiles_x = (Wc + kPyrTile - 1) / kPyrTile;
+  const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
+  const int t = threadIdx.x;
+  // level 0 and 1: each thread a 2 x 2 block of cells
+  {
+    const int y1 = t / 16, x1 = t % 16;
+    const int cy = ty * kPyrTile + 2 * y1, cx = tx * kPyrTile + 2 * x1;
+    if (cy < Hc && cx < Wc) {
+      PyrNode k[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int y = cy + (i >> 1), x = cx + (i & 1);
+        if (y >= Hc || x >= Wc) continue;
+        k[i] = pyramid_leaf_node(o.depth, W, y, x);
+        pyramid_store(o, 0, y, x, k[i]);
+        if (o.prev) {  // each cell saves its lower-left vertex; the last row and column their others
+          const size_t v = (size_t)y * W + x;
+          o.prev[v] = o.depth[v];
+          const bool last_x = x == Wc - 1, last_y = y == Hc - 1;
+          if (last_x) o.prev[v + 1] = o.depth[v + 1];
+          if (last_y) o.prev[v + W] = o.depth[v + W];
+          if (last_x && last_y) o.prev[v + W + 1] = o.depth[v + W + 1];
+        }
+      }
+      if (o.levels > 1) {
+        const PyrNode n = pyramid_up_node([&](int dy, int dx) { return k[2 * dy + dx]; }, Wc, Hc, 1, cy >> 1, cx >> 1,
+                                          Wc, Hc);
+        pyramid_store(o, 1, cy >> 1, cx >> 1, n);
+        s_n[0][y1 * 16 + x1] = n;
+      }
     }
   }
-  pmin[i] = lo;
-  pmax[i] = hi;
+  for (int l = 2; l < kPyrTileLevels && l < o.levels; ++l) {
+    __syncthreads();
+    const int side = kPyrTile >> l, cs = 2 * side;
+    if (t < side * side) {
+      const int ly = t / side, lx = t % side;
+      const int y = ty * side + ly, x = tx * side + lx;
+      if (y < o.lh[l] && x < o.lw[l]) {
+        const PyrNode *c = s_n[l & 1];
+        const PyrNode n = pyramid_up_node([&](int dy, int dx) { return c[(2 * ly + dy) * cs + 2 * lx + dx]; },
+                                          o.lw[l - 1], o.lh[l - 1], l, y, x, Wc, Hc);
+        pyramid_store(o, l, y, x, n);
+        s_n[(l & 1) ^ 1][ly * side + lx] = n;
+      }
+    }
+  }
 }
 
-__global__ void k_pyramid_leaf(const float *__restrict__ depth, int H, int W, float *__restrict__ pmin,
-                               float *__restrict__ pmax) {
-  const int Wc = W - 1, Hc = H - 1;
-  const int n = Wc * Hc;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    pyramid_leaf_node(depth, W, Wc, i, pmin, pmax);
+// Levels 6 and up (one block); children read back from memory, their slack taken off again (rounded up).
+__device__ __forceinline__ void pyramid_top(const PyrObj &o) {
+  const float fw = (float)o.W, fh = (float)o.H;
+  for (int l = kPyrTileLevels; l < o.levels; ++l) {
+    const int w = o.lw[l], n = w * o.lh[l], cw = o.lw[l - 1], co = o.off[l - 1];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const int y = i / w, x = i - y * w;
+      const PyrNode nd = pyramid_up_node(
+          [&](int dy, int dx) {
+            const int j = co + (2 * y + dy) * cw + 2 * x + dx;
+            PyrNode k;
+            k.mx = o.pmax[j];
+            plane_unpack(o.planes[j], k.gx, k.gy, k.c);
+            k.c = __fsub_ru(k.c, plane_slack(k.gx, k.gy, fw, fh));
+            return k;
+          },
+          cw, o.lh[l - 1], l, y, x, o.W - 1, o.H - 1);
+      pyramid_store(o, l, y, x, nd);
+    }
+    __syncthreads();
+  }
 }
 
-__global__ void k_pyramid_up(const float *__restrict__ cmin, const float *__restrict__ cmax, int cw, int ch,
-                             float *__restrict__ pmin, float *__restrict__ pmax, int w, int h) {
-  const int n = w * h;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    pyramid_up_node(cmin, cmax, cw, ch, w, i, pmin, pmax);
+__global__ void __launch_bounds__(kPyrThreads) k_pyramid_tiles(const __grid_constant__ PyrObj o) {
+  pyramid_tile(o, blockIdx.x);
 }
+__global__ void __launch_bounds__(1024) k_pyramid_top(const __grid_constant__ PyrObj o) { pyramid_top(o); }
 
-// Batched pyramid level l over many objects: object o owns the blocks
-// [blk[l] of o, blk[l] of o + 1) of the launch (none once its levels run out).
-__global__ void k_pyramid_b(const PyrObj *__restrict__ objs, int n, int l) {
+// Batched: object o owns the blocks [blk of o, blk of o + 1) of the tile launch, and one block of the top one.
+__global__ void __launch_bounds__(kPyrThreads) k_pyramid_tiles_b(const PyrObj *__restrict__ objs, int n) {
   __shared__ int s_o;
   if (threadIdx.x == 0) {
     int lo = 0, hi = n - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (objs[mid].blk[l] <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+      if (objs[mid].blk <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
     }
     s_o = lo;
   }
   __syncthreads();
   const PyrObj &o = objs[s_o];
-  if (l >= o.levels) return;
-  const int i = ((int)blockIdx.x - o.blk[l]) * blockDim.x + threadIdx.x;
-  if (i >= o.lw[l] * o.lh[l]) return;
-  if (l == 0) {
-    const int W = o.W, Wc = W - 1;
-    pyramid_leaf_node(o.depth, W, Wc, i, o.pmin, o.pmax);
-    if (o.prev) {  // each cell saves its lower-left vertex; the last row and column their others
-      const int cy = i / Wc, cx = i - cy * Wc;
-      const size_t v = (size_t)cy * W + cx;
-      o.prev[v] = o.depth[v];
-      const bool last_x = cx == Wc - 1, last_y = cy == o.H - 2;
-      if (last_x) o.prev[v + 1] = o.depth[v + 1];
-      if (last_y) o.prev[v + W] = o.depth[v + W];
-      if (last_x && last_y) o.prev[v + W + 1] = o.depth[v + W + 1];
-    }
-  } else
-    pyramid_up_node(o.pmin + o.off[l - 1], o.pmax + o.off[l - 1], o.lw[l - 1], o.lh[l - 1], o.lw[l], i,
-                    o.pmin + o.off[l], o.pmax + o.off[l]);
+  pyramid_tile(o, (int)blockIdx.x - o.blk);
+}
+__global__ void __launch_bounds__(1024) k_pyramid_top_b(const PyrObj *__restrict__ objs) {
+  pyramid_top(objs[blockIdx.x]);
+}
+
+int pyramid_tiles(int H, int W) {
+  return ((W - 2 + kPyrTile) / kPyrTile) * ((H - 2 + kPyrTile) / kPyrTile);
 }
 
 void fill_pyr_obj(const Ctx &c, PyrObj &o) {
@@ -97,40 +194,35 @@ void fill_pyr_obj(const Ctx &c, PyrObj &o) {
   o.hz_blk = 0;
   o.depth = c.depth;
   o.prev = c.depth_prev;
-  o.pmin = c.pmin;
   o.pmax = c.pmax;
+  o.planes = c.planes;
   o.H = c.H;
   o.W = c.W;
   o.levels = c.levels;
+  o.blk = 0;
   for (int l = 0; l < kMaxLevels; ++l) {
     o.off[l] = c.off[l];
     o.lw[l] = c.lw[l];
     o.lh[l] = c.lh[l];
-    o.blk[l] = 0;
   }
 }
 
-// One launch per level; blocks[l] = total blocks of level l (objects' ranges set in d_objs).
-cudaError_t build_pyramid_batch(cudaStream_t s, const PyrObj *d_objs, int n, int levels, const int *blocks) {
-  for (int l = 0; l < levels; ++l)
-    if (blocks[l] > 0) k_pyramid_b<<<blocks[l], kPyrThreads, 0, s>>>(d_objs, n, l);
+// blocks: tiles of all objects (their ranges set in d_objs); levels: the most of an object.
+cudaError_t build_pyramid_batch(cudaStream_t s, const PyrObj *d_objs, int n, int levels, int blocks) {
+  k_pyramid_tiles_b<<<blocks, kPyrThreads, 0, s>>>(d_objs, n);
+  if (levels > kPyrTileLevels) k_pyramid_top_b<<<n, 1024, 0, s>>>(d_objs);
   return cudaGetLastError();
 }
 
 cudaError_t build_pyramid(Ctx &c) {
-  const int Wc = c.W - 1, Hc = c.H - 1;
-  const int threads = 256;
-  int blocks = (Wc * Hc + threads - 1) / threads;
-  blocks = blocks < 1 ? 1 : (blocks > 4096 ? 4096 : blocks);
-  k_pyramid_leaf<<<blocks, threads, 0, c.stream>>>(c.depth, c.H, c.W, c.pmin, c.pmax);
-  c.stats.launches += c.levels;
-  for (int l = 1; l < c.levels; ++l) {
-    const int n = c.lw[l] * c.lh[l];
-    int b = (n + threads - 1) / threads;
-    b = b > 4096 ? 4096 : b;
-    k_pyramid_up<<<b, threads, 0, c.stream>>>(c.pmin + c.off[l - 1], c.pmax + c.off[l - 1], c.lw[l - 1],
-                                               c.lh[l - 1], c.pmin + c.off[l], c.pmax + c.off[l], c.lw[l],
-                                               c.lh[l]);
+  PyrObj o;
+  fill_pyr_obj(c, o);
+  o.prev = nullptr;
+  k_pyramid_tiles<<<pyramid_tiles(c.H, c.W), kPyrThreads, 0, c.stream>>>(o);
+  ++c.stats.launches;
+  if (c.levels > kPyrTileLevels) {
+    k_pyramid_top<<<1, 1024, 0, c.stream>>>(o);
+    ++c.stats.launches;
   }
   return cudaGetLastError();
 }
@@ -352,7 +444,9 @@ constexpr int kTraceThreads = 128;
 constexpr int kMarchKeep = IRTPS_MARCH_KEEP;
 // run leaf steps once kLeafBatch * (lanes waiting for one) >= lanes doing node steps
 constexpr int kLeafBatch = IRTPS_LEAF_BATCH;
-enum : int { PH_SETUP = 0, PH_MARCH = 1, PH_RESOLVE = 2, PH_DONE = 3 };
+enum : int { PH_SETUP = 0, PH_MARCH = 1, PH_RESOLVE = 2, PH_DONE = 3, PH_LEAF = 4 };
+// march-loop iterations between two looks at the lanes' step budgets
+constexpr int kMarchMost = 1 << 16;
 
 // Dynamic shared memory of a trace launch over n objects: level tables and item ranges.
 static size_t trace_smem_bytes(int n) { return (size_t)n * sizeof(LevelTable) + (size_t)(n + 1) * sizeof(unsigned); }
@@ -432,7 +526,8 @@ __global__ void __launch_bounds__(kTraceThreads,
     const float *l = ob->lights + 3 * kk;
     return F3{__ldg(l), __ldg(l + 1), __ldg(l + 2)};
   };
-  auto budget0 = [&]() -> int { return 8 * (ob->f.Wc + ob->f.Hc + 8) * (ob->f.levels + 1); };
+  // march-loop iterations a segment may take (a lane waiting for its leaf step counts them too)
+  auto budget0 = [&]() -> int { return 32 * (ob->f.Wc + ob->f.Hc + 8) * (ob->f.levels + 1); };
   const uint32_t iter_base = a.iter_dev ? *a.iter_dev : a.iter;
 
   int phase = alive ? PH_SETUP : PH_DONE;
@@ -456,11 +551,19 @@ __global__ void __launch_bounds__(kTraceThreads,
     thr(c) = 1.0f;
     acc(c) = sum(c) = comp(c) = 0.0f;
   }
+  // the true origin of the current segment (read by leaf and resolve steps only)
+  __shared__ float s_org[3][kTraceThreads];
+  auto org = [&]() -> F3 { return F3{s_org[0][threadIdx.x], s_org[1][threadIdx.x], s_org[2][threadIdx.x]}; };
+  auto set_org = [&](F3 o) {
+    s_org[0][threadIdx.x] = o.x;
+    s_org[1][threadIdx.x] = o.y;
+    s_org[2][threadIdx.x] = o.z;
+  };
   Walker m;
-  bool at_leaf = false;
   bool seen = false;  // per-light item: some sample's first segment hit the surface
   Work w;
   uint32_t segs = 0;
+  unsigned long long visits = 0;  // visits: node steps of the whole warp (the same in every lane)
   int overflow = 0;
 
   // records: per light {hit, visibility} per bounce; light-shared {hit, V_0 .. V_{K-1}} per bounce
@@ -497,7 +600,7 @@ __global__ void __launch_bounds__(kTraceThreads,
     phase = PH_SETUP;
   };
   // after a hit at pixel q (qp) the next bounce starts from the lifted hit point,
-  // which the walker keeps as its origin m.o until the next set-up
+  // kept as the segment origin until the next set-up
   auto continue_path = [&](int q) {
 #pragma unroll
     for (int c = 0; c < C; ++c) thr(c) *= albedo_at(c, q);
@@ -518,11 +621,11 @@ __global__ void __launch_bounds__(kTraceThreads,
       if (f3dot(nq, l) > 0.0f) {
         cosv = fmaxf(0.0f, nq.x * l.x + nq.y * l.y + nq.z * l.z);
         if (ob->shadow) {
-          walker_init(m, m.o, F3{rmul(l.x, ob->Wf), rmul(l.y, ob->Wf), l.z}, true, lt->zmax_margin);
+          phase = walker_init(m, ob->f, *lt, org(), F3{rmul(l.x, ob->Wf), rmul(l.y, ob->Wf), l.z}, true) ? PH_RESOLVE
+                                                                                                      : PH_LEAF;
           shadow = true;
           ++segs;
           budget = budget0();
-          phase = PH_MARCH;
           return;
         }
         if (a.rec) rec_slot(b)[1 + ks] = 1;
@@ -585,28 +688,33 @@ __global__ void __launch_bounds__(kTraceThreads,
           make_uint4((uint32_t)p, (uint32_t)s, (lf << 8) | ((uint32_t)b << 4) | a.stream, ob->iter0 + iter_base),
           ob->key);
       // bounce 1 leaves the pixel's own vertex about its normal; later bounces the
-      // previous hit point (m.o) about the hit pixel's normal
-      const F3 org = b == 1 ? pixel_origin() : m.o;
+      // previous hit point about the hit pixel's normal
+      if (b == 1) set_org(pixel_origin());
+      const F3 o = org();
       const float4 n4 = __ldg(ob->nrm + (b == 1 ? p : qp));
       const F3 dw = cosine_dir(F3{n4.x, n4.y, n4.z}, x.x, x.y);
       const F3 dg = {rmul(dw.x, ob->Wf), rmul(dw.y, ob->Wf), dw.z};
-      walker_init(m, org, dg, false, lt->zmax_margin);
+      // a segment's first cell holds its origin on the surface: it goes straight to the leaf step
+      const bool out = walker_init(m, ob->f, *lt, o, dg, false);
       shadow = false;
       ++segs;
       ++w.draws;
-      phase = PH_MARCH;
-      // early escape: a rising primary ray steeper than the pixel's horizon in its octant
-      // misses everything beyond its first cell; that cell gets its own triangle test
-      if (b == 1 && ob->hz && dg.z > 0.0f && dg.x != 0.0f && dg.y != 0.0f) {
-        const float slope = dg.z / sqrtf(dg.x * dg.x + dg.y * dg.y);
-        const float hz = __ldg(ob->hz + (size_t)octant_of(dg.x, dg.y) * ob->hz_stride + p);
-        if (slope > hz + 1e-5f * fabsf(hz) + 1e-7f) {
-          if ((unsigned)m.cx >= (unsigned)ob->f.Wc || (unsigned)m.cy >= (unsigned)ob->f.Hc) {
-            phase = PH_RESOLVE;  // leaves the grid at once
-          } else {
-            test_cell(ob->f, m.cy, m.cx, m.o, m.d, m.bt, m.btri, w);
-            if (m.btri < 0) phase = PH_RESOLVE;
-            else m.bt = __int_as_float(0x7f800000), m.btri = -1;  // a hit there: the plain march decides
+      phase = out ? PH_RESOLVE : PH_LEAF;
+      if (b == 1 && !out && dg.x != 0.0f && dg.y != 0.0f) {
+        // quick start: a primary ray that leaves its first cell for certain skips that cell's test
+        const int W = ob->f.W, px = p + (m.mx | 1), py = (m.my | 1) * W;
+        const float *h = ob->f.depth;
+        const float hp = __ldg(h + p);
+        if (start_cell_clear(m, rsub(o.z, hp), rsub(__ldg(h + px), hp), rsub(__ldg(h + p + py), hp),
+                             rsub(__ldg(h + px + py), hp))) {
+          walker_cross(m, m.ax, m.ay, lt->top);  // from a vertex, the cell's lines lie at 1 * (1/d)
+          phase = PH_MARCH;
+          // early escape: a rising primary ray steeper than the pixel's horizon in its octant
+          // misses everything beyond its first cell
+          if (ob->hz && dg.z > 0.0f) {
+            const float slope = dg.z / sqrtf(dg.x * dg.x + dg.y * dg.y);
+            const float hz = __ldg(ob->hz + (size_t)octant_of(dg.x, dg.y) * ob->hz_stride + p);
+            if (slope > hz + 1e-5f * fabsf(hz) + 1e-7f) phase = PH_RESOLVE;
           }
         }
       }
@@ -615,25 +723,39 @@ __global__ void __launch_bounds__(kTraceThreads,
     if (live == 0u) break;
     // ---- march while enough of the live lanes are marching; node steps every
     // iteration, leaf steps once enough marching lanes wait for one ----
+    const int n_live = __popc(live);
+    int iters = 0;
     while (true) {
-      if (phase == PH_MARCH && !at_leaf) {
-        if (walker_node_step(m, ob->f, *lt, w, at_leaf)) phase = PH_RESOLVE;
+      const unsigned node = __ballot_sync(0xffffffffu, phase == PH_MARCH);
+      const unsigned leaf = __ballot_sync(0xffffffffu, phase == PH_LEAF);
+      int n_node = __popc(node);
+      const int n_leaf = __popc(leaf);
+      if (n_node + n_leaf == 0 || (kMarchKeep * (n_node + n_leaf) <= n_live && iters > 0) || iters >= kMarchMost) break;
+      ++iters;
+      if (kLeafBatch * n_leaf >= n_node) {
+        if (phase == PH_LEAF) {
+          phase = PH_MARCH;
+          if (walker_leaf_step(m, ob->f, org(), lt->top, w) && walker_finish_walk(m, ob->f, org())) phase = PH_RESOLVE;
+        }
+        n_node = __popc(__ballot_sync(0xffffffffu, phase == PH_MARCH));
       }
-      const unsigned leaf = __ballot_sync(0xffffffffu, phase == PH_MARCH && at_leaf);
-      const unsigned node = __ballot_sync(0xffffffffu, phase == PH_MARCH && !at_leaf);
-      if (leaf != 0u && kLeafBatch * __popc(leaf) >= __popc(node)) {
-        if (phase == PH_MARCH && at_leaf) {
-          at_leaf = false;
-          if (walker_leaf_step(m, ob->f, w)) phase = PH_RESOLVE;
+      visits += n_node;
+      if (phase == PH_MARCH) {
+        bool at_leaf = false;
+        if (walker_node_step(m, BATCH ? lt->planes : a.one.f.planes, *lt, lt->top, at_leaf)) {
+          if (walker_finish_walk(m, ob->f, org())) phase = PH_RESOLVE;
+        } else if (at_leaf) {
+          phase = PH_LEAF;
         }
       }
-      if (phase == PH_MARCH && --budget < 0) {
+    }
+    // a segment that has used up its iterations ends without a hit (counted, an error of the call)
+    if (phase == PH_MARCH || phase == PH_LEAF) {
+      budget -= iters;
+      if (budget < 0) {
         overflow = 1;
-        at_leaf = false;
         phase = PH_RESOLVE;
       }
-      const unsigned marching = __ballot_sync(0xffffffffu, phase == PH_MARCH);
-      if (marching == 0u || kMarchKeep * __popc(marching) <= __popc(live)) break;
     }
     // ---- resolve finished segments ----
     if (phase == PH_RESOLVE) {
@@ -654,7 +776,8 @@ __global__ void __launch_bounds__(kTraceThreads,
         }
       } else if (m.btri < 0) {
         // escaped: environment radiance along the (world) direction
-        const F3 dw = {m.d.x / ob->Wf, m.d.y / ob->Wf, m.d.z};
+        const F3 dg = walker_dir(m);
+        const F3 dw = {dg.x / ob->Wf, dg.y / ob->Wf, dg.z};
         float e[C];
         env_lookup<C>(ob->env, ob->EH, ob->EW, dw, e);
 #pragma unroll
@@ -669,9 +792,11 @@ __global__ void __launch_bounds__(kTraceThreads,
         const int W = ob->f.W, H = ob->f.H;
         const float t = m.bt;
         if (b == 1) seen = true;
-        const F3 q = {radd(m.o.x, rmul(t, m.d.x)), radd(m.o.y, rmul(t, m.d.y)), radd(m.o.z, rmul(t, m.d.z))};
+        const F3 o = org(), d = walker_dir(m);
+        const F3 q = {radd(o.x, rmul(t, d.x)), radd(o.y, rmul(t, d.y)), radd(o.z, rmul(t, d.z))};
         qp = nearest_index(q.y, H) * W + nearest_index(q.x, W);
         const F3 o2 = {q.x, q.y, radd(q.z, ob->eps)};
+        set_org(o2);  // of the shadow rays and of the next bounce
         if (a.rec) {
           int32_t *r = rec_slot(b);
           r[0] = qp;
@@ -679,7 +804,6 @@ __global__ void __launch_bounds__(kTraceThreads,
           for (int i = 1; i < n; ++i) r[i] = -1;
         }
         if constexpr (SHARED) {
-          m.o = o2;  // origin of the shadow rays and of the next bounce
           ks = 0;
           next_light();
         } else {
@@ -689,19 +813,18 @@ __global__ void __launch_bounds__(kTraceThreads,
           if (f3dot(nq, l) > 0.0f) {
             cosv = fmaxf(0.0f, nq.x * l.x + nq.y * l.y + nq.z * l.z);
             if (ob->shadow) {
-              walker_init(m, o2, F3{rmul(l.x, ob->Wf), rmul(l.y, ob->Wf), l.z}, true, lt->zmax_margin);
+              phase = walker_init(m, ob->f, *lt, o2, F3{rmul(l.x, ob->Wf), rmul(l.y, ob->Wf), l.z}, true) ? PH_RESOLVE
+                                                                                                         : PH_LEAF;
               shadow = true;
               ++segs;
-              phase = PH_MARCH;
+              budget = budget0();
             } else {
               if (a.rec) rec_slot(b)[1] = 1;
 #pragma unroll
               for (int c = 0; c < C; ++c) acc(c) = fmaf(thr(c) * albedo_at(c, qp), cosv, acc(c));
-              m.o = o2;
               continue_path(qp);
             }
           } else {
-            m.o = o2;
             continue_path(qp);
           }
         }
@@ -709,11 +832,10 @@ __global__ void __launch_bounds__(kTraceThreads,
     }
   }
   // counters: warp sums, one atomic per warp and counter
-  unsigned long long sg = segs, ov = (unsigned)overflow, nv = w.nodes, tt = w.tris, dr = w.draws;
+  unsigned long long sg = segs, ov = (unsigned)overflow, nv = visits, tt = w.tris, dr = w.draws;
   for (int o = 16; o > 0; o >>= 1) {
     sg += __shfl_down_sync(0xffffffffu, sg, o);
     ov += __shfl_down_sync(0xffffffffu, ov, o);
-    nv += __shfl_down_sync(0xffffffffu, nv, o);
     tt += __shfl_down_sync(0xffffffffu, tt, o);
     dr += __shfl_down_sync(0xffffffffu, dr, o);
   }
