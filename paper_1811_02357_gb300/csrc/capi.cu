@@ -401,7 +401,7 @@ int irtps_create(irtps_ctx **out, int H, int W, int K, int C, const float *light
     c.trace_per_sm_max = c.sms > 0 ? c.trace_blocks / c.sms : 0;
   }
   c.part_stride = c.cg_blocks;
-  if ((rc = dalloc(c, &c.env, (size_t)C * EH * EW, "environment")) ||
+  if ((rc = dalloc(c, &c.env, (size_t)(C == 3 ? 4 : 1) * EH * EW, "environment")) ||
       (rc = dalloc(c, &c.d_lights, (size_t)K * 3, "lights")) ||
       (c.opt.early_escape && H <= 16384 && W <= 16384 &&
        (rc = dalloc(c, &c.horizon, (size_t)8 * P, "horizon bounds"))) ||
@@ -459,7 +459,15 @@ int irtps_create(irtps_ctx **out, int H, int W, int K, int C, const float *light
   }
   e = cudaMallocHost((void **)&c.h_part, sizeof(double) * c.part_stride);
   if (e != cudaSuccess) return bail(cuda_fail(c, e, "create: pinned partials"));
-  e = cudaMemcpyAsync(c.env, env, sizeof(float) * C * EH * EW, cudaMemcpyHostToDevice, c.stream);
+  std::vector<float> texels;  // three channels interleaved as float4
+  if (C == 3) {
+    const size_t n = (size_t)EH * EW;
+    texels.assign(4 * n, 0.0f);
+    for (int ch = 0; ch < 3; ++ch)
+      for (size_t i = 0; i < n; ++i) texels[4 * i + ch] = env[ch * n + i];
+  }
+  e = cudaMemcpyAsync(c.env, C == 3 ? texels.data() : env, sizeof(float) * (C == 3 ? 4 : 1) * EH * EW,
+                      cudaMemcpyHostToDevice, c.stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(c.d_lights, c.h_lights.data(), sizeof(float) * K * 3, cudaMemcpyHostToDevice, c.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.lbar, 0, sizeof(float) * K * C * P, c.stream);

@@ -296,7 +296,8 @@ struct Walker {
                      // a margin), or, rising, above every vertex (plus a margin)
   float bt;
   int btri;
-  int flags;  // bit 0: any-hit; bits 1, 2: a second walk in x, in y; bits 3-4: current walk index
+  int flags;  // bit 0: any-hit; bits 1, 2: a second walk in x, in y; bits 3-4: current walk index; 5-6: see
+              // walker_leaf_step
 };
 
 // The true direction.
@@ -314,18 +315,24 @@ __device__ __forceinline__ float line_e(float k, float s, float o, float inv) {
   return rmul(__fmaf_rn(k, s, -o), inv);
 }
 
+// v moved by one ulp, up or down.
+__device__ __forceinline__ float off_line(float v, bool up) {
+  const int i = __float_as_int(v);
+  if (v == 0.0f) return __int_as_float(up ? 1 : (int)0x80000001);
+  return __int_as_float(i + ((i >= 0) == up ? 1 : -1));
+}
+
 // Start cell of walk `wi` (see above).  Returns false when it lies outside the grid.
 __device__ __forceinline__ bool walker_begin_walk(Walker &m, const Field &f, F3 o, int wi) {
   int cx = (int)floorf(o.x), cy = (int)floorf(o.y);
   if ((float)cx == o.x && m.mx) --cx;
   if ((float)cy == o.y && m.my) --cy;
   if (m.flags & 6) {  // along a grid line: the second walk one column / row back, the origin off the line
-    const int nw = (m.flags & 2) ? 2 : 1;
-    const int wx = wi % nw, wy = wi / nw;
+    const int wx = (m.flags & 2) ? wi & 1 : 0, wy = (m.flags & 2) ? wi >> 1 : wi;
     cx -= wx;
     cy -= wy;
-    if (m.flags & 2) m.ox = nextafterf(o.x, wx ? -INFINITY : INFINITY);
-    if (m.flags & 4) m.oy = nextafterf(o.y, wy ? -INFINITY : INFINITY);
+    if (m.flags & 2) m.ox = off_line(o.x, wx == 0);
+    if (m.flags & 4) m.oy = off_line(o.y, wy == 0);
     m.flags = (m.flags & ~(3 << 3)) | (wi << 3);
   }
   m.nx = cx ^ m.mx;
@@ -335,7 +342,7 @@ __device__ __forceinline__ bool walker_begin_walk(Walker &m, const Field &f, F3 
   return (unsigned)cx < (unsigned)f.Wc && (unsigned)cy < (unsigned)f.Hc;
 }
 
-// Set up a ray.  Returns true when the march is over at once (it starts outside the grid).
+// Set up a ray.  Returns true when its walk is over at once (it starts outside the grid).
 __device__ __forceinline__ bool walker_init(Walker &m, const Field &f, const LevelTable &lt, F3 o, F3 d, bool any) {
   m.mx = d.x < 0.0f ? -1 : 0;
   m.my = d.y < 0.0f ? -1 : 0;
@@ -353,16 +360,14 @@ __device__ __forceinline__ bool walker_init(Walker &m, const Field &f, const Lev
   m.btri = -1;
   // a rising ray is above every vertex (by the margin) beyond this parameter; any rounding of it
   // only moves the end of the walk within the margin, where no triangle can be hit
-  const float t_top = d.z > 0.0f ? (lt.zmax_margin - o.z) / d.z : __int_as_float(0x7f800000);
-  bool in = walker_begin_walk(m, f, o, 0);
-  if (m.flags & 6) {  // skip the walks that start outside the grid
-    const int walks = ((m.flags & 2) ? 2 : 1) * ((m.flags & 4) ? 2 : 1);
-    for (int wi = 1; !in && wi < walks; ++wi) in = walker_begin_walk(m, f, o, wi);
-  }
-  // the grid is left at its far lines' e; te reaching it ends the walk (te > the float below it)
-  const float gx = line_e(m.mx ? 0.0f : (float)f.Wc, 1.0f, m.ox, m.ax);
-  const float gy = line_e(m.my ? 0.0f : (float)f.Hc, 1.0f, m.oy, m.ay);
-  m.t_end = fminf(t_top, __int_as_float(__float_as_int(fminf(gx, gy)) - 1));  // (both e are above 0 when `in`)
+  const float t_top = d.z > 0.0f ? __fdividef(lt.zmax_margin - o.z, d.z) : __int_as_float(0x7f800000);
+  const bool in = walker_begin_walk(m, f, o, 0);
+  // the grid is left at its far lines' e (above 0 when `in`); te reaching it ends the walk (te > the float
+  // below it); an axis along which the ray does not move has none
+  const float inf = __int_as_float(0x7f800000);
+  const float gx = (m.flags & 2) ? inf : line_e(m.mx ? 0.0f : (float)f.Wc, 1.0f, m.ox, m.ax);
+  const float gy = (m.flags & 4) ? inf : line_e(m.my ? 0.0f : (float)f.Hc, 1.0f, m.oy, m.ay);
+  m.t_end = fminf(t_top, __int_as_float(__float_as_int(fminf(gx, gy)) - 1));
   return !in;
 }
 
@@ -376,18 +381,24 @@ __device__ __forceinline__ bool walker_finish_walk(Walker &m, const Field &f, F3
   return true;
 }
 
-// Cross the exit lines at tx, ty (the earlier one; both on a tie) and climb one level when that
-// leaves the parent node (climbing after every skip visits as many nodes but descends twice as often).
+// Cross the exit lines at tx, ty (the earlier one; both on a tie) and climb, by up to kClimb levels, to
+// the largest node whose border that crosses: the bits of the indexes that the step changes say how many
+// levels it leaves.
+#ifndef IRTPS_CLIMB
+#define IRTPS_CLIMB 2
+#endif
+#ifndef IRTPS_START_LEVEL
+#define IRTPS_START_LEVEL 3
+#endif
+constexpr int kClimb = IRTPS_CLIMB;
+constexpr int kStartLevel = IRTPS_START_LEVEL;  // level of a primary ray's march after a quick start
 __device__ __forceinline__ void walker_cross(Walker &m, float tx, float ty, int top) {
-  const bool cx = tx <= ty, cy = ty <= tx;
-  if (cx) ++m.nx;
-  if (cy) ++m.ny;
+  const int nx = m.nx + (tx <= ty ? 1 : 0), ny = m.ny + (ty <= tx ? 1 : 0);
   m.te = fminf(tx, ty);
-  if (((cx && !(m.nx & 1)) || (cy && !(m.ny & 1))) && m.lv < top) {
-    m.nx >>= 1;
-    m.ny >>= 1;
-    ++m.lv;
-  }
+  const int up = min(min(31 - __clz((nx ^ m.nx) | (ny ^ m.ny) | 1), kClimb), top - m.lv);
+  m.nx = nx >> up;
+  m.ny = ny >> up;
+  m.lv += up;
 }
 
 // The march advances in two kinds of steps.  A node step examines the node: it
@@ -400,8 +411,9 @@ __device__ __forceinline__ void walker_cross(Walker &m, float tx, float ty, int 
 // The multiply-adds of the plane test run on the FMA pipes, which the march otherwise leaves idle (the
 // integer and compare pipe is its bound), and the node's edges come from a magic addition.
 __device__ __forceinline__ bool walker_node_step(Walker &m, const uint2 *__restrict__ planes, const LevelTable &lt,
-                                                 int top, bool &at_leaf) {
+                                                 int top, bool &at_leaf, Work &w) {
   if (m.te > m.t_end) return true;
+  ++w.nodes;
   const int2 ol = lt.ol[m.lv];
   const uint2 pv = __ldg(planes + (ol.x + (m.ny ^ m.my) * ol.y + (m.nx ^ m.mx)));
   const float s = __int_as_float(m.lv * (1 << 23) + 0x3f800000);  // 2^lv
@@ -428,47 +440,56 @@ __device__ __forceinline__ bool walker_node_step(Walker &m, const uint2 *__restr
   return false;
 }
 
-// Leaf step: both triangles of the current cell (and, at a near-vertex
-// crossing, of the two cells beside the vertex), then the plain walk's step.
-// Returns true when the walk is over.
-__device__ __forceinline__ bool walker_leaf_step(Walker &m, const Field &f, F3 o, int top, Work &w) {
+// Leaf step: both triangles of the current cell, then the plain walk's step.  At a
+// near-vertex crossing the two cells beside the vertex are tested too, each by a leaf step of
+// its own (flag bits 5-6), so that the test stands in the code once.
+enum : int { LEAF_ON = 0, LEAF_OVER = 1, LEAF_AGAIN = 2 };  // walk on, walk over, another leaf step first
+__device__ __forceinline__ int walker_leaf_step(Walker &m, const Field &f, F3 o, int top, Work &w) {
   const float inf = __int_as_float(0x7f800000);
   const F3 d = walker_dir(m);
-  const int cx = m.nx ^ m.mx, cy = m.ny ^ m.my;
-  test_cell(f, cy, cx, o, d, m.bt, m.btri, w);
+  const int side = (m.flags >> 5) & 3;  // 0: the cell, 1: the one beside it in x, 2: in y
+  const int cx = (m.nx + (side == 1 ? 1 : 0)) ^ m.mx, cy = (m.ny + (side == 2 ? 1 : 0)) ^ m.my;
+  if ((unsigned)cx < (unsigned)f.Wc && (unsigned)cy < (unsigned)f.Hc) test_cell(f, cy, cx, o, d, m.bt, m.btri, w);
   const float tx = line_e(node_edge(m.nx), 1.0f, m.ox, m.ax);
   const float ty = line_e(node_edge(m.ny), 1.0f, m.oy, m.ay);
-  if (tx != inf && ty != inf && fabsf(rsub(tx, ty)) <= rmul(kCorner, fmaxf(tx, ty))) {
-    const int sx = m.mx | 1, sy = m.my | 1;
-    if (cx + sx >= 0 && cx + sx < f.Wc) test_cell(f, cy, cx + sx, o, d, m.bt, m.btri, w);
-    if (cy + sy >= 0 && cy + sy < f.Hc) test_cell(f, cy + sy, cx, o, d, m.bt, m.btri, w);
+  if (fmaxf(tx, ty) < inf && fabsf(rsub(tx, ty)) <= rmul(kCorner, fmaxf(tx, ty)) && side < 2) {
+    m.flags += 1 << 5;
+    return LEAF_AGAIN;
   }
+  m.flags &= ~(3 << 5);
   if (m.btri >= 0) {
-    if (m.flags & 1) return true;
+    if (m.flags & 1) return LEAF_OVER;
     m.t_end = fminf(m.t_end, radd(m.bt, kHitMargin));  // later cells may only hold closer hits
   }
-  if (tx == inf && ty == inf) return true;
+  if (fminf(tx, ty) == inf) return LEAF_OVER;
   walker_cross(m, tx, ty, top);
-  return false;
+  return LEAF_ON;
 }
 
-// One step of either kind, over the walks of a grid-line ray.  Returns true when the march is over.
-__device__ __forceinline__ bool walker_step(Walker &m, const Field &f, const LevelTable &lt, F3 o, Work &w) {
-  bool at_leaf = false;
-  ++w.nodes;
-  bool over = walker_node_step(m, f.planes, lt, f.levels - 1, at_leaf);
-  if (!over && at_leaf) over = walker_leaf_step(m, f, o, f.levels - 1, w);
-  return over && walker_finish_walk(m, f, o);
+// Step over the first cell of a primary ray (it starts at a vertex: the cell's lines lie at 1 * (1/d)), on to
+// level kStartLevel at once: most rays that clear their first cell clear the nodes around it too.
+__device__ __forceinline__ void walker_start_next(Walker &m, int top) {
+  const int lv = min(kStartLevel, top);
+  m.nx = (m.nx + (m.ax <= m.ay ? 1 : 0)) >> lv;
+  m.ny = (m.ny + (m.ay <= m.ax ? 1 : 0)) >> lv;
+  m.te = fminf(m.ax, m.ay);
+  m.lv = lv;
 }
 
 // Blocking march (probes, render): steps until done or until `budget` steps are used.
 __device__ __forceinline__ bool march(const Field &f, const LevelTable &lt, F3 o, F3 d, bool any, float &t, int &tri,
                                      int &budget, Work &w) {
   Walker m;
-  if (!walker_init(m, f, lt, o, d, any)) {
-    while (!walker_step(m, f, lt, o, w)) {
-      if (--budget < 0) break;
+  bool over = walker_init(m, f, lt, o, d, any);
+  while (!(over && walker_finish_walk(m, f, o))) {
+    bool at_leaf = false;
+    over = walker_node_step(m, f.planes, lt, f.levels - 1, at_leaf, w);
+    while (at_leaf) {
+      const int st = walker_leaf_step(m, f, o, f.levels - 1, w);
+      over = st == LEAF_OVER;
+      at_leaf = st == LEAF_AGAIN;
     }
+    if (--budget < 0) break;
   }
   t = m.bt;
   tri = m.btri;

@@ -48,12 +48,13 @@ struct ObjTrace {
   Field f;
   const float4 *nrm;      // H*W (nx, ny, nz, mean albedo)
   const float *albedo;    // C*H*W
-  const float *env;       // C*EH*EW
+  const float *env;       // EH*EW texels: float (one channel) or float4 (three)
   const float *lights;    // K*3, unit, z > 0
   float *out;             // K*C*n_pix
   uint2 key;              // Philox key {seed_lo ^ object, seed_hi}
   int EH, EW, K, spp, bounces, n_pix, shadow;
   float eps, Wf;          // ray-origin lift; W (grid units per world unit in x and y)
+  float inv_w2;           // 1 / W^2
   unsigned item_begin;    // first work item of the object (batched launches)
   uint32_t iter0;         // added to the launch's iteration field
   float *part;            // light-shared sampling: partial sums, n_chunks x n_pix x K x C, then n_chunks x n_pix x C
@@ -109,7 +110,7 @@ struct Ctx {
   size_t shared_cap = 0;          // floats in shared_part
 
   // device buffers (owned)
-  float *env = nullptr;           // C*EH*EW
+  float *env = nullptr;           // EH*EW texels: float (one channel) or float4 (three)
   void *images = nullptr;         // K*C*H*W, float or half
   int images_dtype = IRTPS_F32;
   float *lbar = nullptr;          // K*C*H*W

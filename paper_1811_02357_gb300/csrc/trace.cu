@@ -363,14 +363,17 @@ cudaError_t launch_horizon_batch(cudaStream_t s, const PyrObj *d_objs, int n, in
 // ---------------------------------------------------------------------------
 // Environment: bilinear lookup in a C x EH x EW latitude-longitude map over the
 // full sphere (theta = acos(w_z) down the rows, phi = atan2(w_y, w_x) across,
-// texel centres at half-integers, wrap in phi, clamp in theta).
+// texel centres at half-integers, wrap in phi, clamp in theta), along a grid
+// direction d = (W w_x, W w_y, w_z), inv_w2 = 1 / W^2.  phi needs no division by W.  Three
+// channels are stored as float4 texels: 4 loads a lookup instead of 12.
 // ---------------------------------------------------------------------------
 template <int C>
-__device__ __forceinline__ void env_lookup(const float *__restrict__ env, int EH, int EW, F3 w, float *out) {
-  const float inv = rsqrtf(w.x * w.x + w.y * w.y + w.z * w.z);
-  const float z = fminf(1.0f, fmaxf(-1.0f, w.z * inv));
+__device__ __forceinline__ void env_lookup(const float *__restrict__ env, int EH, int EW, F3 d, float inv_w2,
+                                           float *out) {
+  const float inv = rsqrtf(fmaf(fmaf(d.x, d.x, d.y * d.y), inv_w2, d.z * d.z));
+  const float z = fminf(1.0f, fmaxf(-1.0f, d.z * inv));
   const float theta = acosf(z);
-  float phi = atan2f(w.y, w.x);
+  float phi = atan2f(d.y, d.x);
   if (phi < 0.0f) phi += 6.28318530717958647692f;
   const float row = theta * ((float)EH * 0.318309886183790671538f) - 0.5f;
   const float col = phi * ((float)EW * 0.159154943091895335769f) - 0.5f;
@@ -378,15 +381,25 @@ __device__ __forceinline__ void env_lookup(const float *__restrict__ env, int EH
   const float fr = row - r0, fc = col - c0;
   const int ra = min(EH - 1, max(0, (int)r0));
   const int rb = min(EH - 1, max(0, (int)r0 + 1));
-  int ca = (int)c0 % EW;
+  int ca = (int)c0;  // in -1 .. EW
   if (ca < 0) ca += EW;
+  if (ca >= EW) ca -= EW;
   const int cb = ca + 1 == EW ? 0 : ca + 1;
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    const float *m = env + (size_t)c * EH * EW;
-    const float top = (1.0f - fc) * __ldg(m + ra * EW + ca) + fc * __ldg(m + ra * EW + cb);
-    const float bot = (1.0f - fc) * __ldg(m + rb * EW + ca) + fc * __ldg(m + rb * EW + cb);
-    out[c] = (1.0f - fr) * top + fr * bot;
+  auto mix = [&](float aa, float ab, float ba, float bb) -> float {
+    const float top = (1.0f - fc) * aa + fc * ab;
+    const float bot = (1.0f - fc) * ba + fc * bb;
+    return (1.0f - fr) * top + fr * bot;
+  };
+  if constexpr (C == 3) {
+    const float4 *m = reinterpret_cast<const float4 *>(env);
+    const float4 aa = __ldg(m + ra * EW + ca), ab = __ldg(m + ra * EW + cb);
+    const float4 ba = __ldg(m + rb * EW + ca), bb = __ldg(m + rb * EW + cb);
+    out[0] = mix(aa.x, ab.x, ba.x, bb.x);
+    out[1] = mix(aa.y, ab.y, ba.y, bb.y);
+    out[2] = mix(aa.z, ab.z, ba.z, bb.z);
+  } else {
+    out[0] = mix(__ldg(env + ra * EW + ca), __ldg(env + ra * EW + cb), __ldg(env + rb * EW + ca),
+                 __ldg(env + rb * EW + cb));
   }
 }
 
@@ -434,19 +447,29 @@ struct TraceArgs {
 #define IRTPS_TRACE_MINB_SHARED 9
 #endif
 #ifndef IRTPS_MARCH_KEEP
-#define IRTPS_MARCH_KEEP 2
+#define IRTPS_MARCH_KEEP 4
 #endif
 #ifndef IRTPS_LEAF_BATCH
-#define IRTPS_LEAF_BATCH 4
+#define IRTPS_LEAF_BATCH 2
 #endif
 constexpr int kTraceThreads = 128;
 // leave the march loop when marching lanes <= live lanes / kMarchKeep
 constexpr int kMarchKeep = IRTPS_MARCH_KEEP;
+// set up again before marching while at least this many lanes of the warp have no ray to march
+#ifndef IRTPS_REFILL
+#define IRTPS_REFILL 14
+#endif
+constexpr int kRefill = IRTPS_REFILL;
 // run leaf steps once kLeafBatch * (lanes waiting for one) >= lanes doing node steps
 constexpr int kLeafBatch = IRTPS_LEAF_BATCH;
 enum : int { PH_SETUP = 0, PH_MARCH = 1, PH_RESOLVE = 2, PH_DONE = 3, PH_LEAF = 4 };
 // march-loop iterations between two looks at the lanes' step budgets
 constexpr int kMarchMost = 1 << 16;
+
+// Hides what the compiler knows of a lane's phase, so that it keeps one copy of the code that follows
+// (it otherwise threads each phase's jumps through copies of the next steps, and the warps then wait on
+// instruction fetches).
+__device__ __forceinline__ void keep_apart(int &phase) { asm volatile("" : "+r"(phase)); }
 
 // Dynamic shared memory of a trace launch over n objects: level tables and item ranges.
 static size_t trace_smem_bytes(int n) { return (size_t)n * sizeof(LevelTable) + (size_t)(n + 1) * sizeof(unsigned); }
@@ -460,10 +483,12 @@ __global__ void __launch_bounds__(kTraceThreads,
   const int n_obj = BATCH ? a.n_obj : 1;
   unsigned *s_begin = reinterpret_cast<unsigned *>(lts + n_obj);
   if constexpr (BATCH) {
+#pragma unroll 1
     for (int i = threadIdx.x; i < n_obj * kMaxLevels; i += blockDim.x) {
       const int o = i / kMaxLevels, l = i - o * kMaxLevels;
       lts[o].ol[l] = make_int2(a.objs[o].f.off[l], a.objs[o].f.lw[l]);
     }
+#pragma unroll 1
     for (int o = threadIdx.x; o < n_obj; o += blockDim.x) {
       set_height_bounds(a.objs[o].f, lts + o);
       s_begin[o] = a.objs[o].item_begin;
@@ -475,12 +500,10 @@ __global__ void __launch_bounds__(kTraceThreads,
   // Work items.  Per-light sampling: (object, light k, pixel), within an object
   // item = k * n_pix + ip, all spp samples of (p, k).  Light-shared sampling:
   // (chunk j, pixel), item = j * n_pix + ip, samples [j * chunk, (j + 1) * chunk)
-  // of pixel p for all lights.  Each lane starts with the item of its global
-  // index and, when done, takes the next unclaimed item from a counter (claimed a
-  // warp at a time), so that no lane idles while items remain.  An item is
-  // always traced by one lane, samples in order.
+  // of pixel p for all lights.  A lane without an item takes the next unclaimed
+  // one from a counter (claimed a warp at a time), so that no lane idles while items
+  // remain.  An item is always traced by one lane, samples in order.
   const unsigned n_items = a.n_items;
-  unsigned item = blockIdx.x * blockDim.x + threadIdx.x;
   const ObjTrace *ob = &a.one;
   const LevelTable *lt = lts;
   // the item's indices and the path's bounce state, used at set-up and resolve only, in shared-memory
@@ -488,11 +511,13 @@ __global__ void __launch_bounds__(kTraceThreads,
   __shared__ int s_item[9][kTraceThreads];
   int &k = s_item[0][threadIdx.x], &ip = s_item[1][threadIdx.x], &p = s_item[2][threadIdx.x];
   int &j = s_item[3][threadIdx.x], &s_end = s_item[4][threadIdx.x];
-  k = ip = p = j = s_end = 0;
+  k = p = j = s_end = 0;
+  ip = -1;  // no item yet
+  __shared__ float s_pix[3][kTraceThreads];  // the pixel's own vertex, lifted: origin of the item's primary rays
   auto take = [&](unsigned it) -> int {  // returns the item's first sample
-    item = it;
     if constexpr (BATCH) {
       int lo = 0, hi = n_obj - 1;  // last object whose range starts at or before it
+#pragma unroll 1
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (s_begin[mid] <= it) lo = mid; else hi = mid - 1;
@@ -504,6 +529,10 @@ __global__ void __launch_bounds__(kTraceThreads,
     const int q = (int)(it / (unsigned)ob->n_pix);
     ip = (int)it - q * ob->n_pix;
     p = a.pixels ? a.pixels[ip] : ip;
+    const int pi = p / ob->f.W;
+    s_pix[0][threadIdx.x] = (float)(p - pi * ob->f.W);
+    s_pix[1][threadIdx.x] = (float)pi;
+    s_pix[2][threadIdx.x] = radd(__ldg(ob->f.depth + p), ob->eps);
     if constexpr (SHARED) {
       j = q;
       s_end = min(ob->spp, (j + 1) * ob->chunk);
@@ -513,15 +542,7 @@ __global__ void __launch_bounds__(kTraceThreads,
       return 0;
     }
   };
-  const bool alive = item < n_items;
   int &s = s_item[5][threadIdx.x];
-  s = alive ? take(item) : 0;
-  // the pixel's own vertex, lifted: origin of every primary ray of this lane
-  auto pixel_origin = [&]() -> F3 {
-    const int W = ob->f.W;
-    const int pi = p / W, pj = p - pi * W;
-    return F3{(float)pj, (float)pi, radd(__ldg(ob->f.depth + p), ob->eps)};
-  };
   auto light_k = [&](int kk) -> F3 {
     const float *l = ob->lights + 3 * kk;
     return F3{__ldg(l), __ldg(l + 1), __ldg(l + 2)};
@@ -530,12 +551,13 @@ __global__ void __launch_bounds__(kTraceThreads,
   auto budget0 = [&]() -> int { return 32 * (ob->f.Wc + ob->f.Hc + 8) * (ob->f.levels + 1); };
   const uint32_t iter_base = a.iter_dev ? *a.iter_dev : a.iter;
 
-  int phase = alive ? PH_SETUP : PH_DONE;
+  int phase = PH_SETUP;
+  s = 0x7fffffff;
   int &b = s_item[6][threadIdx.x], &qp = s_item[7][threadIdx.x], &ks = s_item[8][threadIdx.x];
   b = 1;
   qp = 0;
   ks = 0;
-  int budget = alive ? budget0() : 0;
+  int budget = 0;
   bool shadow = false;
   float cosv = 0.0f;
   // the path's throughput and radiance (touched once per segment) and the item's Kahan sums over
@@ -548,8 +570,7 @@ __global__ void __launch_bounds__(kTraceThreads,
   auto comp = [&](int c) -> float & { return s_path[3][c][threadIdx.x]; };
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    thr(c) = 1.0f;
-    acc(c) = sum(c) = comp(c) = 0.0f;
+    sum(c) = comp(c) = 0.0f;
   }
   // the true origin of the current segment (read by leaf and resolve steps only)
   __shared__ float s_org[3][kTraceThreads];
@@ -563,7 +584,6 @@ __global__ void __launch_bounds__(kTraceThreads,
   bool seen = false;  // per-light item: some sample's first segment hit the surface
   Work w;
   uint32_t segs = 0;
-  unsigned long long visits = 0;  // visits: node steps of the whole warp (the same in every lane)
   int overflow = 0;
 
   // records: per light {hit, visibility} per bounce; light-shared {hit, V_0 .. V_{K-1}} per bounce
@@ -584,65 +604,12 @@ __global__ void __launch_bounds__(kTraceThreads,
 #pragma unroll
     for (int c = 0; c < C; ++c) d[c] += thr(c) * albedo_at(c, qp) * cosv;
   };
-  auto end_sample = [&]() {
-#pragma unroll
-    for (int c = 0; c < C; ++c) {  // Kahan summation over samples
-      const float y = acc(c) - comp(c);
-      const float t = sum(c) + y;
-      comp(c) = (t - sum(c)) - y;
-      sum(c) = t;
-      acc(c) = 0.0f;
-      thr(c) = 1.0f;
-    }
-    ++s;
-    b = 1;
-    budget = budget0();
-    phase = PH_SETUP;
-  };
-  // after a hit at pixel q (qp) the next bounce starts from the lifted hit point,
-  // kept as the segment origin until the next set-up
-  auto continue_path = [&](int q) {
-#pragma unroll
-    for (int c = 0; c < C; ++c) thr(c) *= albedo_at(c, q);
-    if (b < ob->bounces) {
-      ++b;
-      phase = PH_SETUP;
-    } else {
-      end_sample();
-    }
-  };
-  // light-shared: the next light from ks on that faces the hit normal gets its
-  // shadow ray (or, without shadow rays, its direct term); then the path goes on
-  auto next_light = [&]() {
-    const float4 m4 = __ldg(ob->nrm + qp);
-    const F3 nq = {m4.x, m4.y, m4.z};
-    while (ks < ob->K) {
-      const F3 l = light_k(ks);
-      if (f3dot(nq, l) > 0.0f) {
-        cosv = fmaxf(0.0f, nq.x * l.x + nq.y * l.y + nq.z * l.z);
-        if (ob->shadow) {
-          phase = walker_init(m, ob->f, *lt, org(), F3{rmul(l.x, ob->Wf), rmul(l.y, ob->Wf), l.z}, true) ? PH_RESOLVE
-                                                                                                      : PH_LEAF;
-          shadow = true;
-          ++segs;
-          budget = budget0();
-          return;
-        }
-        if (a.rec) rec_slot(b)[1 + ks] = 1;
-        add_direct(ks);
-      }
-      ++ks;
-    }
-    shadow = false;
-    continue_path(qp);
-  };
-
   while (true) {
     // ---- finished items: store the result and claim the next item ----
     const bool item_done = phase == PH_SETUP && s >= (SHARED ? s_end : ob->spp);
     const unsigned need = __ballot_sync(0xffffffffu, item_done);
     if (need) {
-      if (item_done) {
+      if (item_done && ip >= 0) {
         if constexpr (SHARED) {
           // the environment part, common to every light, in the item's own C sums
           // (after all chunks' light sums); the reduction adds it to each light
@@ -662,63 +629,71 @@ __global__ void __launch_bounds__(kTraceThreads,
       const int lane = threadIdx.x & 31;
       const int leader = __ffs(need) - 1;
       unsigned base = 0;
-      // the counter counts claims beyond the lanes' start items (one per thread of the grid)
-      if (lane == leader) base = atomicAdd(a.next_item, (unsigned)__popc(need)) + gridDim.x * blockDim.x;
+      if (lane == leader) base = atomicAdd(a.next_item, (unsigned)__popc(need));
       base = __shfl_sync(0xffffffffu, base, leader);
       if (item_done) {
         const unsigned mine = base + (unsigned)__popc(need & ((1u << lane) - 1u));
         if (mine < n_items) {
           s = take(mine);
           b = 1;
-          budget = budget0();
         } else {
           phase = PH_DONE;
         }
       }
     }
-    // ---- set up the next primary or bounce segment ----
+    keep_apart(phase);
+    // ---- set up the next segment: sampled (primary or bounce), or a shadow ray (one code path for both, since
+    // the kernel waits on its instruction fetches: a second set-up inlined cost more than the divergence) ----
     if (phase == PH_SETUP) {
-      if (a.rec && b == 1) {
+      const bool primary = b == 1 && !shadow;
+      if (a.rec && primary) {
         int32_t *r = rec_slot(1);
         const int n = rec_width() * ob->bounces;
+#pragma unroll 1
         for (int i = 0; i < n; ++i) r[i] = -2;
       }
-      const uint32_t lf = SHARED ? 0u : (uint32_t)k;
-      const uint4 x = philox4x32_10(
-          make_uint4((uint32_t)p, (uint32_t)s, (lf << 8) | ((uint32_t)b << 4) | a.stream, ob->iter0 + iter_base),
-          ob->key);
-      // bounce 1 leaves the pixel's own vertex about its normal; later bounces the
-      // previous hit point about the hit pixel's normal
-      if (b == 1) set_org(pixel_origin());
+      F3 dw;
+      if (shadow) {
+        dw = light_k(SHARED ? ks : k);
+      } else {
+        const uint32_t lf = SHARED ? 0u : (uint32_t)k;
+        const uint4 x = philox4x32_10(
+            make_uint4((uint32_t)p, (uint32_t)s, (lf << 8) | ((uint32_t)b << 4) | a.stream, ob->iter0 + iter_base),
+            ob->key);
+        // bounce 1 leaves the pixel's own vertex about its normal; later bounces the
+        // previous hit point about the hit pixel's normal
+        if (primary) set_org(F3{s_pix[0][threadIdx.x], s_pix[1][threadIdx.x], s_pix[2][threadIdx.x]});
+        const float4 n4 = __ldg(ob->nrm + (primary ? p : qp));
+        dw = cosine_dir(F3{n4.x, n4.y, n4.z}, x.x, x.y);
+        ++w.draws;
+      }
       const F3 o = org();
-      const float4 n4 = __ldg(ob->nrm + (b == 1 ? p : qp));
-      const F3 dw = cosine_dir(F3{n4.x, n4.y, n4.z}, x.x, x.y);
       const F3 dg = {rmul(dw.x, ob->Wf), rmul(dw.y, ob->Wf), dw.z};
       // a segment's first cell holds its origin on the surface: it goes straight to the leaf step
-      const bool out = walker_init(m, ob->f, *lt, o, dg, false);
-      shadow = false;
+      const bool out = walker_init(m, ob->f, *lt, o, dg, shadow);
       ++segs;
-      ++w.draws;
+      budget = budget0();
       phase = out ? PH_RESOLVE : PH_LEAF;
-      if (b == 1 && !out && dg.x != 0.0f && dg.y != 0.0f) {
+      if (primary && !out && dg.x != 0.0f && dg.y != 0.0f) {
         // quick start: a primary ray that leaves its first cell for certain skips that cell's test
         const int W = ob->f.W, px = p + (m.mx | 1), py = (m.my | 1) * W;
         const float *h = ob->f.depth;
         const float hp = __ldg(h + p);
         if (start_cell_clear(m, rsub(o.z, hp), rsub(__ldg(h + px), hp), rsub(__ldg(h + p + py), hp),
                              rsub(__ldg(h + px + py), hp))) {
-          walker_cross(m, m.ax, m.ay, lt->top);  // from a vertex, the cell's lines lie at 1 * (1/d)
+          walker_start_next(m, lt->top);
           phase = PH_MARCH;
           // early escape: a rising primary ray steeper than the pixel's horizon in its octant
           // misses everything beyond its first cell
           if (ob->hz && dg.z > 0.0f) {
-            const float slope = dg.z / sqrtf(dg.x * dg.x + dg.y * dg.y);
+            const float slope = dg.z * rsqrtf(dg.x * dg.x + dg.y * dg.y);  // to 2^-21, inside the test's margin
             const float hz = __ldg(ob->hz + (size_t)octant_of(dg.x, dg.y) * ob->hz_stride + p);
             if (slope > hz + 1e-5f * fabsf(hz) + 1e-7f) phase = PH_RESOLVE;
           }
         }
       }
     }
+    keep_apart(phase);
     const unsigned live = __ballot_sync(0xffffffffu, phase != PH_DONE);  // no lane finishes inside the march loop
     if (live == 0u) break;
     // ---- march while enough of the live lanes are marching; node steps every
@@ -728,26 +703,24 @@ __global__ void __launch_bounds__(kTraceThreads,
     while (true) {
       const unsigned node = __ballot_sync(0xffffffffu, phase == PH_MARCH);
       const unsigned leaf = __ballot_sync(0xffffffffu, phase == PH_LEAF);
-      int n_node = __popc(node);
-      const int n_leaf = __popc(leaf);
-      if (n_node + n_leaf == 0 || (kMarchKeep * (n_node + n_leaf) <= n_live && iters > 0) || iters >= kMarchMost) break;
+      const int n_node = __popc(node), n_leaf = __popc(leaf);
+      if (n_node + n_leaf == 0 || iters >= kMarchMost ||
+          (iters > 0 ? kMarchKeep * (n_node + n_leaf) <= n_live : n_live - (n_node + n_leaf) >= kRefill))
+        break;
       ++iters;
       if (kLeafBatch * n_leaf >= n_node) {
         if (phase == PH_LEAF) {
-          phase = PH_MARCH;
-          if (walker_leaf_step(m, ob->f, org(), lt->top, w) && walker_finish_walk(m, ob->f, org())) phase = PH_RESOLVE;
+          const int st = walker_leaf_step(m, ob->f, org(), lt->top, w);
+          phase = st == LEAF_ON ? PH_MARCH : (st == LEAF_OVER ? PH_RESOLVE : PH_LEAF);
         }
-        n_node = __popc(__ballot_sync(0xffffffffu, phase == PH_MARCH));
+        keep_apart(phase);
       }
-      visits += n_node;
       if (phase == PH_MARCH) {
         bool at_leaf = false;
-        if (walker_node_step(m, BATCH ? lt->planes : a.one.f.planes, *lt, lt->top, at_leaf)) {
-          if (walker_finish_walk(m, ob->f, org())) phase = PH_RESOLVE;
-        } else if (at_leaf) {
-          phase = PH_LEAF;
-        }
+        if (walker_node_step(m, BATCH ? lt->planes : a.one.f.planes, *lt, lt->top, at_leaf, w)) phase = PH_RESOLVE;
+        if (at_leaf) phase = PH_LEAF;
       }
+      keep_apart(phase);
     }
     // a segment that has used up its iterations ends without a hit (counted, an error of the call)
     if (phase == PH_MARCH || phase == PH_LEAF) {
@@ -758,36 +731,43 @@ __global__ void __launch_bounds__(kTraceThreads,
       }
     }
     // ---- resolve finished segments ----
+    if (phase == PH_RESOLVE && (m.flags & 6) && !walker_finish_walk(m, ob->f, org()))
+      phase = PH_MARCH;  // a ray along a grid line walks on beside it
     if (phase == PH_RESOLVE) {
+      bool on = false;      // the path goes on to its next bounce
+      bool ended = false;   // the path is over, its radiance in v
+      bool lights = false;  // light-shared: go on with the lights from ks
+      float v[C];
       if (shadow) {
         const int vis = m.btri >= 0 ? 0 : 1;
+        shadow = false;
         if constexpr (SHARED) {
           if (a.rec) rec_slot(b)[1 + ks] = vis;
           if (vis) add_direct(ks);
           ++ks;
-          next_light();
+          lights = true;
         } else {
           if (a.rec) rec_slot(b)[1] = vis;
           if (vis) {
 #pragma unroll
             for (int c = 0; c < C; ++c) acc(c) = fmaf(thr(c) * albedo_at(c, qp), cosv, acc(c));
           }
-          continue_path(qp);
+          on = true;
         }
       } else if (m.btri < 0) {
         // escaped: environment radiance along the (world) direction
-        const F3 dg = walker_dir(m);
-        const F3 dw = {dg.x / ob->Wf, dg.y / ob->Wf, dg.z};
-        float e[C];
-        env_lookup<C>(ob->env, ob->EH, ob->EW, dw, e);
+        env_lookup<C>(ob->env, ob->EH, ob->EW, walker_dir(m), ob->inv_w2, v);
+        if (b > 1) {
 #pragma unroll
-        for (int c = 0; c < C; ++c) acc(c) = fmaf(thr(c), e[c], acc(c));
+          for (int c = 0; c < C; ++c) v[c] = fmaf(thr(c), v[c], acc(c));
+        }
         if (a.rec) {
           int32_t *r = rec_slot(b);
           const int n = rec_width();
+#pragma unroll 1
           for (int i = 0; i < n; ++i) r[i] = -1;
         }
-        end_sample();
+        ended = true;
       } else {
         const int W = ob->f.W, H = ob->f.H;
         const float t = m.bt;
@@ -795,47 +775,97 @@ __global__ void __launch_bounds__(kTraceThreads,
         const F3 o = org(), d = walker_dir(m);
         const F3 q = {radd(o.x, rmul(t, d.x)), radd(o.y, rmul(t, d.y)), radd(o.z, rmul(t, d.z))};
         qp = nearest_index(q.y, H) * W + nearest_index(q.x, W);
-        const F3 o2 = {q.x, q.y, radd(q.z, ob->eps)};
-        set_org(o2);  // of the shadow rays and of the next bounce
+        set_org(F3{q.x, q.y, radd(q.z, ob->eps)});  // of the shadow rays and of the next bounce
+        if (b == 1) {  // the path's first hit: throughput 1, no radiance yet
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            thr(c) = 1.0f;
+            acc(c) = 0.0f;
+          }
+        }
         if (a.rec) {
           int32_t *r = rec_slot(b);
           r[0] = qp;
           const int n = rec_width();
+#pragma unroll 1
           for (int i = 1; i < n; ++i) r[i] = -1;
         }
         if constexpr (SHARED) {
           ks = 0;
-          next_light();
+          lights = true;
         } else {
           const float4 m4 = __ldg(ob->nrm + qp);
           const F3 nq = {m4.x, m4.y, m4.z};
           const F3 l = light_k(k);
+          on = true;
           if (f3dot(nq, l) > 0.0f) {
             cosv = fmaxf(0.0f, nq.x * l.x + nq.y * l.y + nq.z * l.z);
             if (ob->shadow) {
-              phase = walker_init(m, ob->f, *lt, o2, F3{rmul(l.x, ob->Wf), rmul(l.y, ob->Wf), l.z}, true) ? PH_RESOLVE
-                                                                                                         : PH_LEAF;
               shadow = true;
-              ++segs;
-              budget = budget0();
+              phase = PH_SETUP;
+              on = false;
             } else {
               if (a.rec) rec_slot(b)[1] = 1;
 #pragma unroll
               for (int c = 0; c < C; ++c) acc(c) = fmaf(thr(c) * albedo_at(c, qp), cosv, acc(c));
-              continue_path(qp);
             }
-          } else {
-            continue_path(qp);
           }
         }
       }
+      if (SHARED && lights) {
+        // the next light from ks on that faces the hit normal gets its shadow ray (or, without
+        // shadow rays, its direct term); then the path goes on
+        const float4 m4 = __ldg(ob->nrm + qp);
+        const F3 nq = {m4.x, m4.y, m4.z};
+        on = true;
+#pragma unroll 1
+        for (; ks < ob->K; ++ks) {
+          const F3 l = light_k(ks);
+          if (!(f3dot(nq, l) > 0.0f)) continue;
+          cosv = fmaxf(0.0f, nq.x * l.x + nq.y * l.y + nq.z * l.z);
+          if (ob->shadow) {
+            shadow = true;
+            phase = PH_SETUP;
+            on = false;
+            break;
+          }
+          if (a.rec) rec_slot(b)[1 + ks] = 1;
+          add_direct(ks);
+        }
+      }
+      if (on) {
+        phase = PH_SETUP;
+        if (b < ob->bounces) {
+#pragma unroll
+          for (int c = 0; c < C; ++c) thr(c) *= albedo_at(c, qp);
+          ++b;
+        } else {
+#pragma unroll
+          for (int c = 0; c < C; ++c) v[c] = acc(c);
+          ended = true;
+        }
+      }
+      if (ended) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {  // Kahan summation over samples
+          const float y = v[c] - comp(c);
+          const float t = sum(c) + y;
+          comp(c) = (t - sum(c)) - y;
+          sum(c) = t;
+        }
+        ++s;
+        b = 1;
+        phase = PH_SETUP;
+      }
     }
+    keep_apart(phase);
   }
   // counters: warp sums, one atomic per warp and counter
-  unsigned long long sg = segs, ov = (unsigned)overflow, nv = visits, tt = w.tris, dr = w.draws;
+  unsigned long long sg = segs, ov = (unsigned)overflow, nv = w.nodes, tt = w.tris, dr = w.draws;
   for (int o = 16; o > 0; o >>= 1) {
     sg += __shfl_down_sync(0xffffffffu, sg, o);
     ov += __shfl_down_sync(0xffffffffu, ov, o);
+    nv += __shfl_down_sync(0xffffffffu, nv, o);
     tt += __shfl_down_sync(0xffffffffu, tt, o);
     dr += __shfl_down_sync(0xffffffffu, dr, o);
   }
@@ -884,6 +914,7 @@ void fill_obj_trace(const Ctx &c, ObjTrace &o) {
   o.shadow = c.opt.shadow_rays;
   o.eps = c.eps;
   o.Wf = (float)c.W;
+  o.inv_w2 = 1.0f / ((float)c.W * (float)c.W);
   o.item_begin = 0;
   o.iter0 = 0;
   o.part = nullptr;
