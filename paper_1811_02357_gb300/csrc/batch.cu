@@ -125,8 +125,11 @@ int irls_kernels(const irtps_batch &b) {
   return b.irls_iters > 0 ? b.irls_iters * (1 + (b.mg_levels - 1) + 7) + 1 : 0;
 }
 
-// Kernels of the least-squares solve: seven, plus the six transform passes when some object solves directly.
-int solve_kernels(const irtps_batch &b) { return 7 + (b.spectral.n > 0 ? 6 : 0); }
+// Kernels of the least-squares solve: the iterative solve's seven unless every object solves directly, and the
+// transform passes when some object does.
+int solve_kernels(const irtps_batch &b) {
+  return (b.spectral.n < b.n ? 7 : 0) + irtps::spectral_batch_kernels(b.spectral);
+}
 
 // Trace descriptors for this call: objects of larger per-item cost first, so
 // that the cheap items of the last claims fill the tail of the launch.
@@ -477,7 +480,7 @@ int irtps_batch_create(irtps_batch **out, irtps_ctx *const *objs, int n_obj, int
   {
     std::vector<Ctx *> cs;
     for (int i = 0; i < n_obj; ++i) cs.push_back(&objs[i]->c);
-    if (irtps::spectral_batch_setup(cs, b.spectral) != cudaSuccess) {
+    if (irtps::spectral_batch_setup(cs, b.d_stats, b.spectral) != cudaSuccess) {
       cudaGetLastError();
       return bail(IRTPS_ENOMEM);
     }

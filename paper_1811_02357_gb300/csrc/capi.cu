@@ -46,7 +46,7 @@ void release(Ctx &c) {
   void *bufs[] = {c.env, c.d_lights, c.horizon, c.shared_part, c.images, c.lbar, c.depth, c.depth_prev, c.nrm, c.albedo, c.valid, c.pmax, c.planes,
                   c.cg_x, c.cg_b, c.cg_r, c.cg_z, c.cg_p, c.cg_ap, c.part, c.dstats, c.next_item, c.cg_ctl,
                   c.mg_x0, c.mg_x1, c.mg_b, c.mg_wh, c.mg_wv, c.mg_wh_unit, c.mg_wv_unit, c.iter_dev, c.holes,
-                  c.fill_v, c.fill_w, c.sp_ch, c.sp_cw, c.sp_mu, c.sp_nu, c.sp_t, c.ps_pix, c.ps_mask,
+                  c.fill_v, c.fill_w, c.sp_pool, c.sp_t, c.ps_pix, c.ps_mask,
                   c.ps_rhs, c.ps_count};
   for (void *b : bufs)
     if (b) cudaFree(b);

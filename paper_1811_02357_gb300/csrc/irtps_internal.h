@@ -82,6 +82,37 @@ struct FillPyramid {
   size_t total = 0;
 };
 
+// Plan of a complex FFT of n points: radices of m points (m = n, or Bluestein's convolution length when
+// chirp is set), device tables (see spectral.cu).
+constexpr int kMaxFftStages = 14;
+struct FftPlan {
+  int n, m, stages;
+  int radix[kMaxFftStages];
+  const float2 *tw;      // e^{-2 pi i t / m}, t < m
+  const float2 *half;    // e^{-i pi k / 2n}, k < n
+  const float2 *chirp;   // e^{-i pi i^2 / n}, i < n (null: n is 7-smooth)
+  const float2 *filter;  // DFT of the conjugate chirp, / m
+};
+
+// One direct (spectral) depth solve.
+struct SpecObj {
+  int H, W;
+  double h, tol;
+  float nz_min;
+  const float4 *nrm;
+  float *depth;
+  double *b, *x;         // right-hand side, iterate (H x W)
+  float *t;              // spectrum (H x W)
+  double *part;          // partial sums: row_blocks of |b|^2, row_blocks of x, check_blocks of |r|^2
+  CGCtl *ctl;
+  CGAcc *acc;
+  FftPlan row, col;      // lengths W and H
+  const float *mu, *nu;  // eigenvalues of the columns' and rows' path Laplacians
+  int row_blocks, col_blocks, check_blocks;
+  int col_lines;         // complex lines (pairs of columns) per block of the column pass
+  int blk[3];            // first block in a batched launch: row, column, check passes
+};
+
 struct Ctx {
   int H = 0, W = 0, K = 0, C = 0, EH = 0, EW = 0;
   uint32_t obj = 0;
@@ -104,9 +135,10 @@ struct Ctx {
   uint8_t *holes = nullptr;       // fill_holes: K x H x W, 1 where the last trace saw no surface point
   float *fill_v = nullptr, *fill_w = nullptr;  // fill_holes: pyramid levels >= 1, K C and K per pixel
   FillPyramid fill_py;
-  // spectral depth solve (precond = 2): DCT-II matrices H x H and W x W, path-Laplacian
-  // eigenvalues, one H x W work array (FP64)
-  double *sp_ch = nullptr, *sp_cw = nullptr, *sp_mu = nullptr, *sp_nu = nullptr, *sp_t = nullptr;
+  // spectral depth solve (precond = 2): sizes, plans and eigenvalues; their device tables; the work array
+  SpecObj sp{};
+  void *sp_pool = nullptr;
+  float *sp_t = nullptr;
   size_t shared_cap = 0;          // floats in shared_part
 
   // device buffers (owned)
@@ -230,43 +262,25 @@ cudaError_t launch_trace(Ctx &c, const int32_t *pixels, int n_pix, int spp, int 
 // hole interpolation (holes.cu): pyramid of an H x W image; fill the holes (K x H x W, nonzero = hole)
 // of a K x C x H x W device stack in place, scratch v_scr K C py.total and w_scr K py.total floats
 FillPyramid fill_pyramid(int H, int W);
-// spectral depth solve (spectral.cu): grids up to kSpectralMaxSide on both sides
-constexpr int kSpectralMaxSide = 1024;
+// spectral depth solve (spectral.cu): grids up to kSpectralMaxSide on both sides (a Bluestein line of 4095
+// points takes 139 of the SM's 227 KB of shared memory)
+constexpr int kSpectralMaxSide = 4096;
 bool spectral_fits(int H, int W);
-cudaError_t spectral_setup(Ctx &c);                                 // matrices and work array
-cudaError_t launch_spectral(Ctx &c, const double *b, double *x);   // x = A^+ b, unit weights
+cudaError_t spectral_setup(Ctx &c);   // plans and work array
+cudaError_t launch_spectral(Ctx &c);  // the whole solve: normals -> b, x, depth, residual check
 // whether a context's unit-weight solves are direct (option precond = 2 on a grid the transform covers)
 inline bool direct_solve(const Ctx &c) { return c.opt.precond == 2 && c.sp_t != nullptr; }
-// pass descriptors of the direct solve (one 16 x 16 output tile per block)
-struct DctFwd {
-  int M, N, K, L;
-  const double *A;
-  int lda;
-  const double *B;
-  int ldb;
-  double *D;
-  int ldd, dro, dco;
-  const double *mu, *nu;
-  int tiles_n, blk_begin;  // tiles along N; first block of the object in a batched launch
-};
-struct DctInv {
-  int M, N, K1, K2, M2, N2, L;
-  const double *A1, *A2;
-  int lda1, lda2;
-  const double *B1, *B2;
-  int ldb1, ldb2;
-  double *D;
-  int ldd;
-  int tiles_n, blk_begin;
-};
-// the direct solves of a batch's objects: six pass tables (four forward, two inverse) in one device block
+// the direct solves of a batch's objects: descriptors in one device table
 struct SpectralBatch {
-  int n = 0;          // objects with direct solves
-  int blocks[6] = {0};
+  int n = 0;              // objects with direct solves
+  int blocks[3] = {0};    // row, column, check passes
+  int refine = 0;         // refinement steps
+  size_t row_smem = 0, col_smem = 0;
   void *table = nullptr;  // owned
 };
-cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, SpectralBatch &sb);
+cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, SpectralBatch &sb);
 cudaError_t launch_spectral_batch(cudaStream_t s, const SpectralBatch &sb);
+int spectral_batch_kernels(const SpectralBatch &sb);
 cudaError_t launch_interpolate_holes(cudaStream_t s, float *values, const uint8_t *holes, int K, int C,
                                      const FillPyramid &py, float *v_scr, float *w_scr, int sms, int &launches);
 cudaError_t launch_next_iter(Ctx &c);  // iter_dev += 1 (end of a captured iteration)

@@ -889,40 +889,18 @@ __global__ void __launch_bounds__(kThreads) k_mg_coarsen(const MG m, int l, floa
   mg_coarsen_body(m, l, wh, wv, whole_grid());
 }
 
-// A direct (spectral) solve counts as one iteration; its FP64 residual is checked
-// against the tolerance like the last one of a PCG loop.
-__global__ void k_direct_done(const CGCtl *ctl, CGAcc *acc, double tol) {
-  const double rel = ctl->rel;
-  acc->iters += 1;
-  acc->last_iters = 1;
-  acc->rel_last = rel;
-  if (!isfinite(ctl->bnorm) || !isfinite(rel) || rel > tol) acc->bad = 1;
-}
-
 // One depth solve, enqueued without host round trips: right-hand side, warm
 // start, residual, |b| on the device, the cooperative PCG loop, mean removal.
 // Unit-weight solves with precond = 2 take the direct cosine-transform solve
-// instead of the loop, then the same residual check and mean removal.
+// (spectral.cu) instead, with the same residual check.
 template <bool WEIGHTED>
 static cudaError_t solve_once(Ctx &c) {
+  if (!WEIGHTED && direct_solve(c)) return launch_spectral(c);
   const CG g = make_cg(c);
   const int nb = c.cg_blocks;
   CGCtl *ctl = (CGCtl *)c.cg_ctl;
   CGAcc *acc = &c.dstats->cg;
   k_rhs<WEIGHTED><<<nb, kThreads, 0, c.stream>>>(g);
-  if (!WEIGHTED && c.opt.precond == 2 && c.sp_t) {
-    LAUNCH_CHECK();
-    cudaError_t e = launch_spectral(c, c.cg_b, c.cg_x);
-    if (e != cudaSuccess) return e;
-    k_residual<false><<<nb, kThreads, 0, c.stream>>>(g, S_RZ0);
-    k_cg_start<<<1, 32, 0, c.stream>>>(g, ctl);
-    k_direct_done<<<1, 1, 0, c.stream>>>(ctl, acc, c.opt.cg_tol);
-    k_sum_x<<<nb, kThreads, 0, c.stream>>>(g);
-    k_store_depth<<<nb, kThreads, 0, c.stream>>>(g, ctl);
-    c.stats.launches += 6;
-    LAUNCH_CHECK();
-    return cudaSuccess;
-  }
   k_load_x<<<nb, kThreads, 0, c.stream>>>(g);
   k_residual<WEIGHTED><<<nb, kThreads, 0, c.stream>>>(g, S_RZ0);
   k_cg_start<<<1, 32, 0, c.stream>>>(g, ctl);
@@ -1002,7 +980,7 @@ struct CGJob {
   const float *old;  // previous surface (D_H)
   double tol;
   int max_iter, check, pre;
-  int direct;      // unit-weight solves by the cosine transform (their passes run before the loop)
+  int direct;      // unit-weight solves by the cosine transform (they skip the iterative solve)
   int blk_begin;
   // robust integration (IRLS): the object's writable level-0.. weights, their unit copy, threshold
   float *wh, *wv;
@@ -1033,7 +1011,9 @@ __device__ __forceinline__ void for_team(const CGJob *__restrict__ jobs, int n, 
 
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads) k_rhs_b(const CGJob *jobs, int n) {
-  for_team(jobs, n, [](const CGJob &j, Team t) { rhs_body<WEIGHTED>(j.g, t); });
+  for_team(jobs, n, [](const CGJob &j, Team t) {
+    if (WEIGHTED || !j.direct) rhs_body<WEIGHTED>(j.g, t);
+  });
 }
 // the warm start of the iterative solves (a direct solve has its x already)
 template <bool WEIGHTED>
@@ -1044,35 +1024,36 @@ __global__ void __launch_bounds__(kThreads) k_load_x_b(const CGJob *jobs, int n)
 }
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads) k_residual_b(const CGJob *jobs, int n) {
-  for_team(jobs, n, [](const CGJob &j, Team t) { residual_body<WEIGHTED>(j.g, S_RZ0, t); });
+  for_team(jobs, n, [](const CGJob &j, Team t) {
+    if (WEIGHTED || !j.direct) residual_body<WEIGHTED>(j.g, S_RZ0, t);
+  });
 }
 // one warp per job
-__global__ void k_cg_start_b(const CGJob *jobs) { cg_start_body(jobs[blockIdx.x].g, jobs[blockIdx.x].ctl); }
+template <bool WEIGHTED>
+__global__ void k_cg_start_b(const CGJob *jobs) {
+  if (WEIGHTED || !jobs[blockIdx.x].direct) cg_start_body(jobs[blockIdx.x].g, jobs[blockIdx.x].ctl);
+}
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads, IRTPS_CG_BATCH_MINB) k_cg_loop_b(const CGJob *jobs, int n) {
   for_team<WEIGHTED>(jobs, n, [](const CGJob &j, Team t) {
-    if (!WEIGHTED && j.direct) {  // solved directly: one iteration, its FP64 residual checked
-      if (t.bid == 0 && threadIdx.x == 0) {
-        const double rel = j.ctl->rel;
-        CGAcc *acc = &j.ds->cg;
-        acc->iters += 1;
-        acc->last_iters = 1;
-        acc->rel_last = rel;
-        if (!isfinite(j.ctl->bnorm) || !isfinite(rel) || rel > j.tol) acc->bad = 1;
-      }
-      return;
-    }
+    if (!WEIGHTED && j.direct) return;  // solved by the transform
     if (j.pre == 1)
       cg_loop_body<1, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, t);
     else
       cg_loop_body<0, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, t);
   });
 }
+template <bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads) k_sum_x_b(const CGJob *jobs, int n) {
-  for_team(jobs, n, [](const CGJob &j, Team t) { sum_x_body(j.g, t); });
+  for_team(jobs, n, [](const CGJob &j, Team t) {
+    if (WEIGHTED || !j.direct) sum_x_body(j.g, t);
+  });
 }
+template <bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads) k_store_depth_b(const CGJob *jobs, int n) {
-  for_team(jobs, n, [](const CGJob &j, Team t) { store_depth_body(j.g, j.ctl, t); });
+  for_team(jobs, n, [](const CGJob &j, Team t) {
+    if (WEIGHTED || !j.direct) store_depth_body(j.g, j.ctl, t);
+  });
 }
 __global__ void __launch_bounds__(kThreads) k_depth_change_b(const CGJob *jobs, int n) {
   for_team(jobs, n, [](const CGJob &j, Team t) { depth_change_body(j.g, j.old, t); });
@@ -1141,22 +1122,21 @@ void cg_fill_job(Ctx &c, int nblk, int blk_begin, DevStats *ds, void *dst) {
 
 template <bool WEIGHTED>
 static cudaError_t solve_batch_once(cudaStream_t s, const CGJob *jobs, int n, int blocks, const SpectralBatch &sb) {
-  k_rhs_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
   if (!WEIGHTED) {
-    LAUNCH_CHECK();
     cudaError_t e = launch_spectral_batch(s, sb);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || sb.n == n) return e;  // every object solved directly
   }
+  k_rhs_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
   k_load_x_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
   k_residual_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
-  k_cg_start_b<<<n, 32, 0, s>>>(jobs);
+  k_cg_start_b<WEIGHTED><<<n, 32, 0, s>>>(jobs);
   LAUNCH_CHECK();
   void *args[] = {(void *)&jobs, (void *)&n};
   cudaError_t e =
       cudaLaunchCooperativeKernel((const void *)k_cg_loop_b<WEIGHTED>, dim3(blocks), dim3(kThreads), args, 0, s);
   if (e != cudaSuccess) return e;
-  k_sum_x_b<<<blocks, kThreads, 0, s>>>(jobs, n);
-  k_store_depth_b<<<blocks, kThreads, 0, s>>>(jobs, n);
+  k_sum_x_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
+  k_store_depth_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
   LAUNCH_CHECK();
   return cudaSuccess;
 }

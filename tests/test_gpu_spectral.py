@@ -1,0 +1,59 @@
+"""The direct depth solve (fast cosine transforms in FP32, refined with FP64 residuals) at the lengths where its
+parts meet: every radix, chirp-convolution (prime) lengths, one- to eight-column blocks, odd row and column
+counts, the longest lines; and a batch that mixes direct and iterative solves."""
+import numpy as np
+import pytest
+
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _normals(H, W):
+    rs = np.random.default_rng(H + 5 * W)
+    X, Y = scenes.grid(H, W)
+    gx = 0.6 * np.sin(7 * X) * np.cos(5 * Y) + rs.normal(0, 0.05, (H, W)) + 0.4
+    gy = 0.5 * np.cos(6 * X + 2 * Y) + rs.normal(0, 0.05, (H, W)) - 0.3
+    return scenes.normals_from_gradient(gx, gy).astype(np.float32)
+
+
+def _context(lib, H, W):
+    ctx = lib.Context(H, W, scenes.ring_lights(3, 45.0), np.zeros((1, 2, 2), np.float32))
+    ctx.set_state(depth=np.zeros((H, W), np.float32), normals=_normals(H, W))
+    return ctx
+
+
+@pytest.mark.parametrize("H,W", [(2, 3), (3, 2), (7, 5), (11, 13), (49, 27), (31, 97), (121, 250), (63, 640),
+                                 (1031, 64), (90, 2047), (1500, 1201), (4096, 3), (3, 4093)])
+def test_direct_solve(lib, oracle_mod, H, W):
+    with _context(lib, H, W) as ctx:
+        ctx.integrate()
+        d, st = ctx.depth(), ctx.stats()
+        ctx.integrate()
+        assert np.array_equal(ctx.depth(), d)  # no dependence on the current depth, no run-to-run change
+    want = oracle_mod.poisson_solve(_normals(H, W).astype(np.float64), 1.0 / W)
+    # the stored depth's FP32 rounding (2^-24 of the largest value), and the refined solve well below it
+    assert np.abs(d - want).max() <= 2.0 ** -23 * np.abs(want).max()
+    assert st["cg_iterations"] == 1 and st["cg_rel_residual"] <= 1e-10, st
+
+
+def test_batch_mixes_direct_and_iterative(lib):
+    sizes = [(40, 44), (2, 4100), (33, 70)]
+    rs = np.random.default_rng(3)
+    images = [rs.uniform(0.2, 0.6, (3, 1, H, W)).astype(np.float32) for H, W in sizes]
+    lights, env = scenes.ring_lights(3, 45.0), np.full((1, 2, 2), 0.1, np.float32)
+    single = []
+    for (H, W), a in zip(sizes, images):
+        with lib.Context(H, W, lights, env) as ctx:
+            ctx.set_images(a)
+            single.append((ctx.depth(), ctx.stats()["cg_iterations"]))
+    ctxs = [lib.Context(H, W, lights, env) for H, W in sizes]
+    with lib.Batch(ctxs) as b:
+        b.set_images(images)
+        got = [c.depth() for c in ctxs]
+    for c in ctxs:
+        c.close()
+    assert [s[1] == 1 for s in single] == [True, False, True]
+    for i in (0, 2):
+        assert np.array_equal(got[i], single[i][0])
+    assert np.abs(got[1] - single[1][0]).max() <= 1e-4 * np.ptp(single[1][0])
