@@ -22,6 +22,7 @@ struct irtps_batch {
   bool shared = false;  // light-shared sampling (every object's option)
   int irls_iters = 0;   // robust-integration reweighting steps (every object's option)
   int mg_levels = 0;    // most multigrid levels of an object
+  size_t cg_smem = 0;   // weighted spectral solves: dynamic shared memory of a solver block
   int use_graph = 0;
   cudaStream_t stream = nullptr;      // where the batch's work runs
   cudaStream_t own_stream = nullptr;
@@ -122,7 +123,8 @@ int trace_grid(const irtps_batch &b) { return b.trace_per_sm * b.sms; }
 
 // Kernels the robust-integration steps add to each batched solve.
 int irls_kernels(const irtps_batch &b) {
-  return b.irls_iters > 0 ? b.irls_iters * (1 + (b.mg_levels - 1) + 7) + 1 : 0;
+  const bool mg = b.spectral.n < b.n;  // some object's weighted solves take the multigrid hierarchy
+  return b.irls_iters > 0 ? b.irls_iters * (1 + (mg ? b.mg_levels - 1 : 0) + 7) + (mg ? 1 : 0) : 0;
 }
 
 // Kernels of the least-squares solve: the iterative solve's seven unless every object solves directly, and the
@@ -233,7 +235,8 @@ int enqueue_iteration(irtps_batch &b, uint32_t iter, bool captured) {
   BCK(irtps::launch_ps_batch(b.stream, b.C, b.objs[0]->c.images_dtype, b.d_ps, b.n, b.ps_blocks), "ps launch");
   BSTAGE(ST_PS, false);
   BSTAGE(ST_DEPTH, true);
-  BCK(irtps::solve_depth_batch_async(b.stream, b.d_jobs, b.n, b.cg_blocks, b.irls_iters, b.mg_levels, b.spectral), "depth solve launch");
+  BCK(irtps::solve_depth_batch_async(b.stream, b.d_jobs, b.n, b.cg_blocks, b.irls_iters, b.mg_levels, b.spectral,
+                                      b.cg_smem), "depth solve launch");
   BSTAGE(ST_DEPTH, false);
   BCK(irtps::depth_change_batch_async(b.stream, b.d_jobs, b.n, b.cg_blocks), "depth change launch");
   if (captured) BCK(irtps::launch_next_iter(b.stream, b.iter_dev), "iteration counter");
@@ -449,7 +452,10 @@ int irtps_batch_create(irtps_batch **out, irtps_ctx *const *objs, int n_obj, int
   }
   // depth solves: every object gets a team, the co-resident grid shared in
   // proportion to the pixel counts (at most the object's own solve grid)
-  const int budget = irtps::cg_batch_grid_limit();
+  if (b.irls_iters > 0)
+    for (int i = 0; i < n_obj; ++i)
+      if (irtps::direct_solve(objs[i]->c)) b.cg_smem = std::max(b.cg_smem, irtps::spec_line_smem(objs[i]->c));
+  const int budget = irtps::cg_batch_grid_limit(b.cg_smem);
   if (budget < n_obj) return bail(IRTPS_ECUDA);
   double total_p = 0.0;
   for (int i = 0; i < n_obj; ++i) total_p += (double)objs[i]->c.H * objs[i]->c.W;
@@ -521,7 +527,8 @@ int irtps_batch_set_images(irtps_batch *x, const void *const *images, int dtype,
   BSTAGE(ST_PS, false);
   BSTAGE(ST_DEPTH, true);
   BCK(irtps::zero_depth_batch_async(b.stream, b.d_jobs, b.n, b.cg_blocks), "depth reset");
-  BCK(irtps::solve_depth_batch_async(b.stream, b.d_jobs, b.n, b.cg_blocks, b.irls_iters, b.mg_levels, b.spectral), "depth solve launch");
+  BCK(irtps::solve_depth_batch_async(b.stream, b.d_jobs, b.n, b.cg_blocks, b.irls_iters, b.mg_levels, b.spectral,
+                                      b.cg_smem), "depth solve launch");
   BSTAGE(ST_DEPTH, false);
   b.primary_per_iter = 0;
   rc = end_call(b, true, 0, nullptr);

@@ -267,6 +267,8 @@ FillPyramid fill_pyramid(int H, int W);
 constexpr int kSpectralMaxSide = 4096;
 bool spectral_fits(int H, int W);
 cudaError_t spectral_setup(Ctx &c);   // plans and work array
+SpecObj spec_object(const Ctx &c, CGAcc *acc);
+size_t spec_line_smem(const Ctx &c);  // shared memory of one line pair, rows or columns
 cudaError_t launch_spectral(Ctx &c);  // the whole solve: normals -> b, x, depth, residual check
 // whether a context's unit-weight solves are direct (option precond = 2 on a grid the transform covers)
 inline bool direct_solve(const Ctx &c) { return c.opt.precond == 2 && c.sp_t != nullptr; }
@@ -325,9 +327,9 @@ int cg_grid_limit();  // co-resident blocks available to the cooperative solve
 // batched solves: one job per object, teams of blocks in one launch per step
 size_t cg_job_bytes();
 void cg_fill_job(Ctx &c, int nblk, int blk_begin, DevStats *ds, void *dst);
-int cg_batch_grid_limit();
+int cg_batch_grid_limit(size_t smem);  // smem: dynamic shared memory of a block (weighted spectral solves)
 cudaError_t solve_depth_batch_async(cudaStream_t s, const void *d_jobs, int n, int blocks, int irls_iters,
-                                    int max_levels, const SpectralBatch &sb);
+                                    int max_levels, const SpectralBatch &sb, size_t smem);
 cudaError_t depth_change_batch_async(cudaStream_t s, const void *d_jobs, int n, int blocks);
 cudaError_t zero_depth_batch_async(cudaStream_t s, const void *d_jobs, int n, int blocks);
 void mg_layout(int H, int W, int *levels, int *h, int *w, int *off, int *total);

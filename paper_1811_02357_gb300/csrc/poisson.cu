@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "irtps_internal.h"
+#include "spectral.cuh"
 
 namespace irtps {
 
@@ -466,8 +467,30 @@ __device__ void mg_vcycle(const MG &m, const float *r, CGCtl *ctl, Team t) {
 }
 #undef MG_FOR
 
+// z = A_1^+ r by the FP32 cosine transforms (A_1 the unit-weight Laplacian), a preconditioner of the weighted
+// solves: the Huber weights lie in (0, 1] and differ from 1 at a tenth of the edges, so PCG takes 16 to 21
+// iterations to 1e-9 whatever the grid, four barriers each, where the V-cycle takes some thirty barriers and
+// several times the iterations.  Called by all blocks with r complete; on return all of z is visible to all blocks.
+__device__ void spectral_solve(const SpecObj &o, const float *r, float *z, CGCtl *ctl, Team t) {
+  for (int i = t.bid; i < o.row_blocks; i += t.nblk) {
+    spec::rows_forward<spec::SRC_ARRAY>(o, i, r);
+    __syncthreads();
+  }
+  grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+  for (int i = t.bid; i < (o.W + 1) / 2; i += t.nblk) {
+    spec::columns(o, i, 1);
+    __syncthreads();
+  }
+  grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+  for (int i = t.bid; i < o.row_blocks; i += t.nblk) {
+    spec::rows_back<spec::DST_ARRAY>(o, i, z);
+    __syncthreads();
+  }
+  grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+}
+
 // The whole PCG loop in one cooperative launch (PRE 0: Jacobi, M = diag(degree);
-// PRE 1: the multigrid V-cycle above).  The iterate is x = x64 + e: the FP64 part
+// PRE 1: the multigrid V-cycle above; PRE 2: the unit-weight spectral solve `so`, weighted solves).  The iterate is x = x64 + e: the FP64 part
 // changes only at a refresh, the FP32 correction e collects alpha * p in between.
 // Per iteration:
 //  A: beta = rz_{it-1}/rz_{it-2}; p_it = z + beta p_{it-1} (also at the 4
@@ -483,7 +506,7 @@ __device__ void mg_vcycle(const MG &m, const float *r, CGCtl *ctl, Team t) {
 // so takes the same decisions.
 template <int PRE, bool WEIGHTED>
 __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc, double tol, int max_iter, int check,
-                                             const MG &mg, Team t) {
+                                             const MG &mg, const SpecObj *so, Team t) {
   __shared__ double sh[33];
   __shared__ float shf[33];
   __shared__ float s_ab[2];
@@ -498,15 +521,14 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
   for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) e[q.p] = 0.0f;
   // z = M^-1 r and the partial sums of r.z into `slot` (and the refresh reference)
   auto precondition = [&](int slot, bool refresh) {
-    if (PRE == 1) {
-      grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);  // r complete
-      mg_vcycle(mg, g.r, ctl, t);
-    }
+    if (PRE != 0) grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);  // r complete
+    if (PRE == 1) mg_vcycle(mg, g.r, ctl, t);
+    if (PRE == 2) spectral_solve(*so, g.r, g.z, ctl, t);
     float rz = 0.0f;
     for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
       const float rf = g.r[q.p];
       float zf;
-      if (PRE == 1) {
+      if (PRE != 0) {
         zf = z[q.p];
       } else {
         zf = WEIGHTED ? rf / weighted_degree(g.wh, g.wv, q.p, q.i, q.j, g.H, g.W)
@@ -521,7 +543,7 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
       if (refresh) g.part[S_RZREF * g.stride + t.bid] = (double)rz;
     }
   };
-  if (PRE == 1 && rel > tol) {  // the residual kernel left r; z and r.z come from the V-cycle
+  if (PRE != 0 && rel > tol) {  // the residual kernel left r; z and r.z come from the preconditioner
     precondition(S_RZ0, true);
     grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
   }
@@ -630,8 +652,15 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
 template <int PRE, bool WEIGHTED = false>
 __global__ void __launch_bounds__(kThreads) k_cg_loop(const CG g, CGCtl *ctl, CGAcc *acc, double tol, int max_iter,
                                                       int check, const MG mg) {
-  cg_loop_body<PRE, WEIGHTED>(g, ctl, acc, tol, max_iter, check, mg, whole_grid());
+  cg_loop_body<PRE, WEIGHTED>(g, ctl, acc, tol, max_iter, check, mg, nullptr, whole_grid());
 }
+__global__ void __launch_bounds__(kThreads) k_cg_loop_spectral(const CG g, CGCtl *ctl, CGAcc *acc, double tol,
+                                                               int max_iter, int check,
+                                                               const __grid_constant__ SpecObj so) {
+  const MG none{};
+  cg_loop_body<2, true>(g, ctl, acc, tol, max_iter, check, none, &so, whole_grid());
+}
+static_assert(kThreads == spec::kSpecThreads, "the spectral passes run in the solver's blocks");
 
 // Start of a solve: |b| and the warm start's relative residual from the partials,
 // barrier state reset (one warp).
@@ -896,8 +925,19 @@ __global__ void __launch_bounds__(kThreads) k_mg_coarsen(const MG m, int l, floa
 template <bool WEIGHTED>
 static cudaError_t solve_once(Ctx &c) {
   if (!WEIGHTED && direct_solve(c)) return launch_spectral(c);
-  const CG g = make_cg(c);
-  const int nb = c.cg_blocks;
+  CG g = make_cg(c);
+  const bool spectral = WEIGHTED && direct_solve(c);
+  const size_t smem = spectral ? spec_line_smem(c) : 0;
+  if (spectral) {  // the cooperative grid that fits with the lines in shared memory
+    cudaError_t e =
+        cudaFuncSetAttribute(k_cg_loop_spectral, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int per = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cg_loop_spectral, kThreads, smem);
+    if (e != cudaSuccess) return e;
+    if (per < 1) return cudaErrorInvalidConfiguration;
+    g.nblk = std::min(g.nblk, per * (c.sms > 0 ? c.sms : 1));
+  }
+  const int nb = g.nblk;
   CGCtl *ctl = (CGCtl *)c.cg_ctl;
   CGAcc *acc = &c.dstats->cg;
   k_rhs<WEIGHTED><<<nb, kThreads, 0, c.stream>>>(g);
@@ -910,10 +950,14 @@ static cudaError_t solve_once(Ctx &c) {
   int max_iter = c.opt.cg_max_iter;
   MG mg = make_mg(c);
   if (WEIGHTED) mg.cscale = 1.0f;
-  void *args[] = {(void *)&g, (void *)&ctl, (void *)&acc, (void *)&tol, (void *)&max_iter, (void *)&m, (void *)&mg};
-  // multigrid for precond 1, and for the solves the spectral form does not cover
-  const void *fn = c.opt.precond != 0 ? (const void *)k_cg_loop<1, WEIGHTED> : (const void *)k_cg_loop<0, WEIGHTED>;
-  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nb), dim3(kThreads), args, 0, c.stream);
+  SpecObj so = spectral ? spec_object(c, acc) : SpecObj{};
+  void *args[] = {(void *)&g, (void *)&ctl, (void *)&acc, (void *)&tol, (void *)&max_iter, (void *)&m,
+                  spectral ? (void *)&so : (void *)&mg};
+  // precond 2: the spectral preconditioner where the transform covers the grid; multigrid elsewhere and for precond 1
+  const void *fn = spectral ? (const void *)k_cg_loop_spectral
+                            : (c.opt.precond != 0 ? (const void *)k_cg_loop<1, WEIGHTED>
+                                                  : (const void *)k_cg_loop<0, WEIGHTED>);
+  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nb), dim3(kThreads), args, smem, c.stream);
   if (e != cudaSuccess) return e;
   k_sum_x<<<nb, kThreads, 0, c.stream>>>(g);
   k_store_depth<<<nb, kThreads, 0, c.stream>>>(g, ctl);
@@ -933,14 +977,18 @@ cudaError_t solve_depth_async(Ctx &c) {
   const int nb = c.cg_blocks;
   for (int it = 0; it < c.opt.irls_iters; ++it) {
     k_irls_weights<<<nb, kThreads, 0, c.stream>>>(g, c.mg_wh, c.mg_wv, (double)c.opt.irls_delta);
-    for (int l = 0; l + 1 < mg.levels; ++l) {
-      const int n = mg.H[l + 1] * mg.W[l + 1];
-      k_mg_coarsen<<<(n + kThreads - 1) / kThreads, kThreads, 0, c.stream>>>(mg, l, c.mg_wh, c.mg_wv);
+    c.stats.launches += 1;
+    if (!direct_solve(c)) {  // the spectral preconditioner needs no hierarchy
+      for (int l = 0; l + 1 < mg.levels; ++l) {
+        const int n = mg.H[l + 1] * mg.W[l + 1];
+        k_mg_coarsen<<<(n + kThreads - 1) / kThreads, kThreads, 0, c.stream>>>(mg, l, c.mg_wh, c.mg_wv);
+      }
+      c.stats.launches += mg.levels - 1;
     }
-    c.stats.launches += mg.levels;
     LAUNCH_CHECK();
     if ((e = solve_once<true>(c)) != cudaSuccess) return e;
   }
+  if (direct_solve(c)) return cudaSuccess;  // unit-weight solves read no weights
   const size_t bytes = sizeof(float) * (size_t)c.mg_total;
   e = cudaMemcpyAsync(c.mg_wh, c.mg_wh_unit, bytes, cudaMemcpyDeviceToDevice, c.stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c.mg_wv, c.mg_wv_unit, bytes, cudaMemcpyDeviceToDevice, c.stream);
@@ -980,7 +1028,9 @@ struct CGJob {
   const float *old;  // previous surface (D_H)
   double tol;
   int max_iter, check, pre;
-  int direct;      // unit-weight solves by the cosine transform (they skip the iterative solve)
+  int direct;      // unit-weight solves by the cosine transform (they skip the iterative solve); weighted ones
+                   // preconditioned by it
+  SpecObj spec;    // direct: the transform's descriptor
   int blk_begin;
   // robust integration (IRLS): the object's writable level-0.. weights, their unit copy, threshold
   float *wh, *wv;
@@ -1037,10 +1087,12 @@ template <bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads, IRTPS_CG_BATCH_MINB) k_cg_loop_b(const CGJob *jobs, int n) {
   for_team<WEIGHTED>(jobs, n, [](const CGJob &j, Team t) {
     if (!WEIGHTED && j.direct) return;  // solved by the transform
-    if (j.pre == 1)
-      cg_loop_body<1, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, t);
+    if (WEIGHTED && j.direct)
+      cg_loop_body<2, true>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, &j.spec, t);
+    else if (j.pre == 1)
+      cg_loop_body<1, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, nullptr, t);
     else
-      cg_loop_body<0, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, t);
+      cg_loop_body<0, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, nullptr, t);
   });
 }
 template <bool WEIGHTED>
@@ -1064,11 +1116,12 @@ __global__ void __launch_bounds__(kThreads) k_irls_weights_b(const CGJob *jobs, 
 }
 __global__ void __launch_bounds__(kThreads) k_mg_coarsen_b(const CGJob *jobs, int n, int l) {
   for_team(jobs, n, [l](const CGJob &j, Team t) {
-    if (l + 1 < j.mg.levels) mg_coarsen_body(j.mg, l, j.wh, j.wv, t);
+    if (!j.direct && l + 1 < j.mg.levels) mg_coarsen_body(j.mg, l, j.wh, j.wv, t);
   });
 }
 __global__ void __launch_bounds__(kThreads) k_unit_weights_b(const CGJob *jobs, int n) {
   for_team(jobs, n, [](const CGJob &j, Team t) {
+    if (j.direct) return;
     for (int q = t.bid * blockDim.x + threadIdx.x; q < j.mg_total; q += t.nblk * blockDim.x) {
       j.wh[q] = j.wh_unit[q];
       j.wv[q] = j.wv_unit[q];
@@ -1084,13 +1137,16 @@ __global__ void __launch_bounds__(kThreads) k_zero_depth_b(const CGJob *jobs, in
 size_t cg_job_bytes() { return sizeof(CGJob); }
 
 // Co-resident blocks of the batched solve loop (at most IRTPS_CG_BATCH_BLOCKS_PER_SM per SM).
-int cg_batch_grid_limit() {
+int cg_batch_grid_limit(size_t smem) {
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
   int per_w = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cg_loop_b<false>, kThreads, 0) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_w, k_cg_loop_b<true>, kThreads, 0) != cudaSuccess) return 0;
+  if (smem > 0 && cudaFuncSetAttribute(k_cg_loop_b<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+                      cudaSuccess)
+    return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_w, k_cg_loop_b<true>, kThreads, smem) != cudaSuccess) return 0;
   per = per < per_w ? per : per_w;
   per = per < IRTPS_CG_BATCH_BLOCKS_PER_SM ? per : IRTPS_CG_BATCH_BLOCKS_PER_SM;
   return per * sms;
@@ -1110,6 +1166,7 @@ void cg_fill_job(Ctx &c, int nblk, int blk_begin, DevStats *ds, void *dst) {
   j.check = c.opt.cg_check_every > 0 ? c.opt.cg_check_every : 10;
   j.pre = c.opt.precond != 0 ? 1 : 0;  // iterative solves: multigrid for precond 1 and 2
   j.direct = direct_solve(c) ? 1 : 0;
+  if (j.direct) j.spec = spec_object(c, &ds->cg);
   j.blk_begin = blk_begin;
   j.wh = c.mg_wh;
   j.wv = c.mg_wv;
@@ -1121,7 +1178,8 @@ void cg_fill_job(Ctx &c, int nblk, int blk_begin, DevStats *ds, void *dst) {
 }
 
 template <bool WEIGHTED>
-static cudaError_t solve_batch_once(cudaStream_t s, const CGJob *jobs, int n, int blocks, const SpectralBatch &sb) {
+static cudaError_t solve_batch_once(cudaStream_t s, const CGJob *jobs, int n, int blocks, const SpectralBatch &sb,
+                                    size_t smem) {
   if (!WEIGHTED) {
     cudaError_t e = launch_spectral_batch(s, sb);
     if (e != cudaSuccess || sb.n == n) return e;  // every object solved directly
@@ -1132,8 +1190,13 @@ static cudaError_t solve_batch_once(cudaStream_t s, const CGJob *jobs, int n, in
   k_cg_start_b<WEIGHTED><<<n, 32, 0, s>>>(jobs);
   LAUNCH_CHECK();
   void *args[] = {(void *)&jobs, (void *)&n};
-  cudaError_t e =
-      cudaLaunchCooperativeKernel((const void *)k_cg_loop_b<WEIGHTED>, dim3(blocks), dim3(kThreads), args, 0, s);
+  if (WEIGHTED && smem > 0) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_cg_loop_b<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_cg_loop_b<WEIGHTED>, dim3(blocks), dim3(kThreads), args,
+                                              WEIGHTED ? smem : 0, s);
   if (e != cudaSuccess) return e;
   k_sum_x_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
   k_store_depth_b<WEIGHTED><<<blocks, kThreads, 0, s>>>(jobs, n);
@@ -1145,17 +1208,18 @@ static cudaError_t solve_batch_once(cudaStream_t s, const CGJob *jobs, int n, in
 // followed by that many reweighting steps of the Huber M-estimator, as in the
 // single-object solve, and the unit weights are put back at the end.
 cudaError_t solve_depth_batch_async(cudaStream_t s, const void *d_jobs, int n, int blocks, int irls_iters,
-                                    int max_levels, const SpectralBatch &sb) {
+                                    int max_levels, const SpectralBatch &sb, size_t smem) {
   const CGJob *jobs = (const CGJob *)d_jobs;
-  cudaError_t e = solve_batch_once<false>(s, jobs, n, blocks, sb);
+  cudaError_t e = solve_batch_once<false>(s, jobs, n, blocks, sb, 0);
   if (e != cudaSuccess || irls_iters <= 0) return e;
   for (int it = 0; it < irls_iters; ++it) {
     k_irls_weights_b<<<blocks, kThreads, 0, s>>>(jobs, n);
-    for (int l = 0; l + 1 < max_levels; ++l) k_mg_coarsen_b<<<blocks, kThreads, 0, s>>>(jobs, n, l);
+    if (sb.n < n)
+      for (int l = 0; l + 1 < max_levels; ++l) k_mg_coarsen_b<<<blocks, kThreads, 0, s>>>(jobs, n, l);
     LAUNCH_CHECK();
-    if ((e = solve_batch_once<true>(s, jobs, n, blocks, sb)) != cudaSuccess) return e;
+    if ((e = solve_batch_once<true>(s, jobs, n, blocks, sb, smem)) != cudaSuccess) return e;
   }
-  k_unit_weights_b<<<blocks, kThreads, 0, s>>>(jobs, n);
+  if (sb.n < n) k_unit_weights_b<<<blocks, kThreads, 0, s>>>(jobs, n);
   LAUNCH_CHECK();
   return cudaSuccess;
 }

@@ -57,3 +57,42 @@ def test_batch_mixes_direct_and_iterative(lib):
     for i in (0, 2):
         assert np.array_equal(got[i], single[i][0])
     assert np.abs(got[1] - single[1][0]).max() <= 1e-4 * np.ptp(single[1][0])
+
+
+@pytest.mark.parametrize("H,W,iters", [(97, 101, 2), (256, 130, 3), (3, 700, 2)])
+def test_weighted_solve_spectral_preconditioner(lib, oracle_mod, H, W, iters):
+    """Robust integration whose weighted solves are preconditioned by the transform, alone and in a batch beside a
+    grid it does not cover, against the oracle's weighted solves (the bar of every weighted solve test)."""
+    n = _normals(H, W)
+    n[H // 2:H // 2 + 3, W // 3:W // 3 + 9] = np.array([0.6, 0.0, 0.8], np.float32)
+    opt = lib.irtps_default_options()
+    opt.irls_iters = iters
+    with lib.Context(H, W, scenes.ring_lights(3, 45.0), np.zeros((1, 2, 2), np.float32), opt) as ctx:
+        ctx.set_state(depth=np.zeros((H, W), np.float32), normals=n)
+        ctx.integrate()
+        d, st = ctx.depth(), ctx.stats()
+    want = oracle_mod.irls_solve(n.astype(np.float64), 1.0 / W, 0.05, iters)
+    assert st["cg_rel_residual"] <= 1e-9 and st["cg_iterations"] <= 60, st
+    assert np.abs(d - want).max() <= 1e-4 * np.ptp(want)
+
+
+def test_weighted_batch_mixes_preconditioners(lib):
+    sizes = [(40, 44), (2, 4100), (33, 70)]
+    rs = np.random.default_rng(4)
+    images = [rs.uniform(0.2, 0.6, (3, 1, H, W)).astype(np.float32) for H, W in sizes]
+    lights, env = scenes.ring_lights(3, 45.0), np.full((1, 2, 2), 0.1, np.float32)
+    opt = lib.irtps_default_options()
+    opt.irls_iters = 2
+    single = []
+    for (H, W), a in zip(sizes, images):
+        with lib.Context(H, W, lights, env, opt) as ctx:
+            ctx.set_images(a)
+            single.append(ctx.depth())
+    ctxs = [lib.Context(H, W, lights, env, opt) for H, W in sizes]
+    with lib.Batch(ctxs) as b:
+        b.set_images(images)
+        got = [c.depth() for c in ctxs]
+    for c in ctxs:
+        c.close()
+    for s, g in zip(single, got):
+        assert np.abs(g - s).max() <= 1e-4 * np.ptp(s)
