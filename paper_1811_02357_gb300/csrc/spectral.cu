@@ -54,14 +54,18 @@ __device__ __forceinline__ void spec_pass(const SpecObj &o, int blk) {
   if (PASS == SP_BACK_LAST) rows_back<DST_ADD_LAST>(o, blk);
   if (PASS == SP_CHECK) check(o, blk, o.check_blocks);
 }
+#ifndef IRTPS_COL_THREADS
+#define IRTPS_COL_THREADS 512
+#endif
+constexpr int kColThreads = IRTPS_COL_THREADS;  // threads of a column block
 template <int PASS>
-__global__ void __launch_bounds__(kSpecThreads) k_spec(const __grid_constant__ SpecObj o) {
+__global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) k_spec(const __grid_constant__ SpecObj o) {
   spec_pass<PASS>(o, blockIdx.x);
 }
 
 // Batched: object i owns the blocks [blk[g] of i, blk[g] of i + 1) of a launch, g = 0 rows, 1 columns, 2 check.
 template <int PASS>
-__global__ void __launch_bounds__(kSpecThreads) k_spec_b(const SpecObj *__restrict__ objs, int n) {
+__global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) k_spec_b(const SpecObj *__restrict__ objs, int n) {
   constexpr int g = PASS == SP_COLS ? 1 : (PASS == SP_CHECK ? 2 : 0);
   __shared__ int s_o;
   if (threadIdx.x == 0) {
@@ -165,9 +169,10 @@ PlanTables make_plan(int n, std::vector<float2> &pool) {
 size_t row_smem(const SpecObj &o) { return sizeof(float2) * 2 * line_stride(o.row.m); }
 size_t col_smem(const SpecObj &o) { return sizeof(float2) * 2 * o.col_lines * line_stride(o.col.m); }
 
-// Solves after which the refinement ends: three pass the default tolerance (1e-9) with two orders of margin
-// on every grid up to 4096 on a side; tighter tolerances get two more, down to the floor of FP64.
-int refinements(double tol) { return tol >= 1e-10 ? 2 : 4; }
+// Refinement steps after the first solve: two pass the default tolerance (1e-9) with two orders of margin on
+// every grid up to 4096 on a side, and one does up to 128 on a side (residual 5e-12 at 64, 3e-11 at 129); tighter
+// tolerances get four, down to the floor of FP64.
+int refinements(const SpecObj &o) { return o.tol < 1e-10 ? 4 : (std::max(o.H, o.W) <= 128 ? 1 : 2); }
 
 template <typename F>
 cudaError_t allow_smem(F *k, size_t bytes) {
@@ -254,12 +259,12 @@ cudaError_t launch_spectral(Ctx &c) {
     return e;
   cudaStream_t s = c.stream;
   k_spec<SP_ROWS_FIRST><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
-  k_spec<SP_COLS><<<o.col_blocks, kSpecThreads, cs, s>>>(o);
+  k_spec<SP_COLS><<<o.col_blocks, kColThreads, cs, s>>>(o);
   k_spec<SP_BACK_FIRST><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
-  const int n = refinements(o.tol);
+  const int n = refinements(o);
   for (int i = 0; i < n; ++i) {
     k_spec<SP_ROWS><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
-    k_spec<SP_COLS><<<o.col_blocks, kSpecThreads, cs, s>>>(o);
+    k_spec<SP_COLS><<<o.col_blocks, kColThreads, cs, s>>>(o);
     if (i + 1 < n)
       k_spec<SP_BACK><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
     else
@@ -286,7 +291,7 @@ cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, S
     sb.blocks[2] += o.check_blocks;
     sb.row_smem = std::max(sb.row_smem, row_smem(o));
     sb.col_smem = std::max(sb.col_smem, col_smem(o));
-    sb.refine = std::max(sb.refine, refinements(o.tol));
+    sb.refine = std::max(sb.refine, refinements(o));
     t.push_back(o);
     ++sb.n;
   }
@@ -311,11 +316,11 @@ cudaError_t launch_spectral_batch(cudaStream_t s, const SpectralBatch &sb) {
       (e = allow_smem(k_spec_b<SP_BACK_LAST>, rs)) != cudaSuccess || (e = allow_smem(k_spec_b<SP_COLS>, cs)) != cudaSuccess)
     return e;
   k_spec_b<SP_ROWS_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
-  k_spec_b<SP_COLS><<<sb.blocks[1], kSpecThreads, cs, s>>>(t, n);
+  k_spec_b<SP_COLS><<<sb.blocks[1], kColThreads, cs, s>>>(t, n);
   k_spec_b<SP_BACK_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
   for (int i = 0; i < sb.refine; ++i) {
     k_spec_b<SP_ROWS><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
-    k_spec_b<SP_COLS><<<sb.blocks[1], kSpecThreads, cs, s>>>(t, n);
+    k_spec_b<SP_COLS><<<sb.blocks[1], kColThreads, cs, s>>>(t, n);
     if (i + 1 < sb.refine)
       k_spec_b<SP_BACK><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
     else

@@ -132,9 +132,13 @@ __device__ __forceinline__ void fft_stage(const float2 *__restrict__ in, float2 
     float2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = in[base + at(j + r * nb)];
-    if (ns > 1) {
+    if (ns > 1) {  // one table load, the other powers by products (a few roundings more, against R - 1 scattered loads)
+      float2 w[R];
+      w[1] = __ldg(tw + k * step);
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(tw + r * k * step));
+      for (int r = 2; r < R; ++r) w[r] = cmul(w[r / 2], w[r - r / 2]);
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], w[r]);
     }
     dft_small<R>(v);
     const int o = q * ns * R + k;
@@ -214,42 +218,49 @@ __device__ __forceinline__ float2 idct_pair(float2 c, float2 cr, float2 w, float
   return make_float2((va.y + vb.x) * scale, (va.x - vb.y) * scale);
 }
 
-// n.x / nz as a FP32 quotient plus the quotient of its exact remainder (48 bits), in FP64.
-__device__ __forceinline__ double quotient(float a, float b) {
-  const float q = __fdiv_rn(a, b);
-  return (double)q + (double)__fdividef(fmaf(-q, b, a), b);
-}
-__device__ __forceinline__ double slope_p(const float4 &n, float nz_min) { return -quotient(n.x, fmaxf(n.z, nz_min)); }
-__device__ __forceinline__ double slope_q(const float4 &n, float nz_min) { return -quotient(n.y, fmaxf(n.z, nz_min)); }
+// A sum of quotients a / b of FP32 numbers to about 48 bits, on the FP32 pipes: each is a FP32 quotient plus the
+// quotient of its exact remainder; the quotients are added with an error-free two-sum.
+struct QuotientSum {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float q = __fdiv_rn(a, b);
+    const float e = __fdividef(__fmaf_rn(-q, b, a), b);
+    const float s = __fadd_rn(hi, q), t = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(q, t)), e));
+    hi = s;
+  }
+};
 
-// Right-hand side b = D^T g of pixel (i, j): trapezoidal edge targets h (s_a + s_b) / 2.
+// Right-hand side b = D^T g of pixel (i, j): trapezoidal edge targets h (s_a + s_b) / 2, slopes -n_x / n_z, -n_y / n_z.
 __device__ __forceinline__ double rhs_at(const SpecObj &o, int i, int j) {
   const float4 *n = o.nrm + (size_t)i * o.W + j;
   const bool l = j > 0, r = j < o.W - 1, u = i > 0, d = i < o.H - 1;
-  double v = 0.0;
-  if (l) v += slope_p(__ldg(n - 1), o.nz_min);
-  if (r) v -= slope_p(__ldg(n + 1), o.nz_min);
-  if (u) v += slope_q(__ldg(n - o.W), o.nz_min);
-  if (d) v -= slope_q(__ldg(n + o.W), o.nz_min);
+  QuotientSum v;
+  auto add = [&](float c, const float4 &m) { v.add(c, fmaxf(m.z, o.nz_min)); };
+  if (l) { const float4 m = __ldg(n - 1); add(-m.x, m); }
+  if (r) { const float4 m = __ldg(n + 1); add(m.x, m); }
+  if (u) { const float4 m = __ldg(n - o.W); add(-m.y, m); }
+  if (d) { const float4 m = __ldg(n + o.W); add(m.y, m); }
   if (l != r || u != d) {  // on a border the pixel's own slope does not cancel
-    const float4 c = __ldg(n);
-    if (l != r) v += l ? slope_p(c, o.nz_min) : -slope_p(c, o.nz_min);
-    if (u != d) v += u ? slope_q(c, o.nz_min) : -slope_q(c, o.nz_min);
+    const float4 m = __ldg(n);
+    if (l != r) add(l ? -m.x : m.x, m);
+    if (u != d) add(u ? -m.y : m.y, m);
   }
-  return 0.5 * o.h * v;
+  return 0.5 * o.h * ((double)v.hi + (double)v.lo);
 }
 
 // r = b - A x of pixel (i, j) in FP64.
 __device__ __forceinline__ double residual_at(const SpecObj &o, int i, int j) {
   const size_t p = (size_t)i * o.W + j;
   const double *x = o.x + p;
-  double s = 0.0;
-  int deg = 0;
-  if (j > 0) { s += x[-1]; ++deg; }
-  if (j < o.W - 1) { s += x[1]; ++deg; }
-  if (i > 0) { s += x[-o.W]; ++deg; }
-  if (i < o.H - 1) { s += x[o.W]; ++deg; }
-  return o.b[p] - fma((double)deg, x[0], -s);
+  if (j > 0 && j < o.W - 1 && i > 0 && i < o.H - 1)  // FP64 is what bounds this: five operations
+    return fma(-4.0, x[0], (x[-1] + x[1]) + (x[-o.W] + x[o.W])) + o.b[p];
+  double s = o.b[p];
+  if (j > 0) s += x[-1] - x[0];
+  if (j < o.W - 1) s += x[1] - x[0];
+  if (i > 0) s += x[-o.W] - x[0];
+  if (i < o.H - 1) s += x[o.W] - x[0];
+  return s;
 }
 
 // Block sum in FP64; the result is valid in thread 0.
@@ -314,13 +325,16 @@ __device__ __forceinline__ void rows_forward(const SpecObj &o, int blk, const fl
 }
 
 // Columns: 2 L columns per block, forward, divided by the eigenvalues, and back.
-__device__ __forceinline__ void columns(const SpecObj &o, int blk, int L) {
+template <int L>
+__device__ __forceinline__ void columns_of(const SpecObj &o, int blk) {
+  constexpr int C = 2 * L;
   const FftPlan &P = o.col;
-  const int n = o.H, W = o.W, C = 2 * L, c0 = blk * C;
+  const int n = o.H, W = o.W, c0 = blk * C;
   const int ls = line_stride(P.m);
   float2 *a = spec_smem, *b = a + L * ls;
+#pragma unroll 4
   for (int e = threadIdx.x; e < n * C; e += blockDim.x) {
-    const int i = e / C, cc = e - i * C;  // C is 2, 4 or 8
+    const int i = e / C, cc = e - i * C;
     const float v = c0 + cc < W ? o.t[(size_t)i * W + c0 + cc] : 0.0f;
     reinterpret_cast<float *>(a + (cc >> 1) * ls + at(place(i, n)))[cc & 1] = v;
   }
@@ -328,7 +342,7 @@ __device__ __forceinline__ void columns(const SpecObj &o, int blk, int L) {
   const float s0 = 1.0f / (float)n;
   const int nk = n / 2 + 1;
   for (int e = threadIdx.x; e < L * nk; e += blockDim.x) {
-    const int l = e / nk, k = e - l * nk, kr = k ? n - k : 0;
+    const int k = e / L, l = e - k * L, kr = k ? n - k : 0;
     float2 *p = z + l * ls + at(k), *pr = z + l * ls + at(kr);
     const float2 zk = *p, zr = *pr;
     const float2 w = __ldg(P.half + k), wr = __ldg(P.half + kr);
@@ -345,11 +359,18 @@ __device__ __forceinline__ void columns(const SpecObj &o, int blk, int L) {
   }
   float2 *y = z == a ? b : a;
   z = dft_lines(P, z, y, L);
+#pragma unroll 4
   for (int e = threadIdx.x; e < n * C; e += blockDim.x) {
     const int i = e / C, cc = e - i * C;
     if (c0 + cc < W)  // swapped: the first line of a pair is in the imaginary part
       o.t[(size_t)i * W + c0 + cc] = reinterpret_cast<const float *>(z + (cc >> 1) * ls + at(place(i, n)))[1 - (cc & 1)];
   }
+}
+
+__device__ __forceinline__ void columns(const SpecObj &o, int blk, int L) {
+  if (L == 4) columns_of<4>(o, blk);
+  else if (L == 2) columns_of<2>(o, blk);
+  else columns_of<1>(o, blk);
 }
 
 // Rows back: two rows per block, into the FP64 iterate (set, or added to; the last one's partial sums give the
@@ -409,14 +430,15 @@ __device__ __forceinline__ void check(const SpecObj &o, int blk, int nblk) {
   if (threadIdx.x == 0) s_mean = rr / (double)P;
   __syncthreads();
   const double mean = s_mean;
-  rr = 0.0;
+  float rf = 0.0f;
   for (int p = blk * blockDim.x + threadIdx.x; p < P; p += nblk * blockDim.x) {
     const int i = p / o.W;
-    const double r = residual_at(o, i, p - i * o.W);
-    rr += r * r;
+    // FP32 squares (a thread's few dozen), scaled clear of underflow: the FP64 pipe bounds this pass
+    const float r = (float)residual_at(o, i, p - i * o.W) * 1.099511627776e12f;  // 2^40
+    rf = fmaf(r, r, rf);
     o.depth[p] = (float)(o.x[p] - mean);
   }
-  rr = block_sum(rr, sh);
+  rr = block_sum((double)rf * 8.271806125530277e-25, sh);  // 2^-80
   double *part = o.part + 2 * o.row_blocks;
   if (threadIdx.x == 0) {
     part[blk] = rr;
