@@ -35,8 +35,9 @@ struct irtps_batch {
   void *d_jobs = nullptr;  // depth-solve jobs
   irtps::SpectralBatch spectral;  // the direct solves of the objects that take them
   irtps::PyrObj *d_pyr = nullptr;
-  irtps::ReduceObj *d_reduce = nullptr;  // light-shared: partial-sum buffers of the objects
-  int reduce_blocks = 0;
+  irtps::ReduceObj *d_reduce = nullptr;  // partial-sum buffers: light-shared of every object, per light of those
+                                         // whose samples are split
+  int reduce_blocks = 0, n_reduce = 0;
   irtps::DevStats *d_stats = nullptr;  // per object (solver, D_H); [n]: trace counters
   unsigned *next_item = nullptr;
   uint32_t *iter_dev = nullptr;
@@ -140,12 +141,12 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
   for (int i = 0; i < b.n; ++i) order[i] = i;
   auto cost = [&](int i) -> long long {  // samples x bounces of one work item (x K when shared)
     const Ctx &c = b.objs[i]->c;
-    if (!b.shared) return (long long)spp[i] * bounces[i];
+    if (!b.shared) return (long long)irtps::light_split(c, spp[i]).chunk * bounces[i];
     return (long long)irtps::shared_split(c.H * c.W, spp[i]).chunk * bounces[i] * c.K;
   };
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
   std::vector<irtps::ObjTrace> h(b.n);
-  std::vector<irtps::ReduceObj> red(b.shared ? b.n : 0);
+  std::vector<irtps::ReduceObj> red;
   unsigned begin = 0;
   unsigned long long primary = 0, items = 0;
   int rblk = 0;
@@ -165,26 +166,29 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
     o.item_begin = begin;
     o.iter0 = c.t;
     unsigned long long n_it = (unsigned long long)P * c.K;
-    if (b.shared) {  // (chunk, pixel) items; partial sums in the object's scratch
-      const irtps::SharedSplit sp = irtps::shared_split(P, spp[i]);
-      o.n_chunks = sp.n_chunks;
-      o.chunk = sp.chunk;
+    // (chunk, pixel) items, or (chunk, light, pixel) items of a small object: partial sums in the object's scratch
+    const irtps::SharedSplit sp = b.shared ? irtps::shared_split(P, spp[i]) : irtps::light_split(c, spp[i]);
+    o.n_chunks = sp.n_chunks;
+    o.chunk = sp.chunk;
+    if (b.shared || sp.n_chunks > 1) {
       bool g = false;
-      BCK(irtps::ensure_shared_scratch(c, (size_t)o.n_chunks * (c.K + 1) * c.C * P, g), "light-shared partial sums");
+      BCK(irtps::ensure_shared_scratch(c, irtps::trace_scratch_floats(c, P, spp[i]), g), "trace partial sums");
       grown = grown || g;
       o.part = c.shared_part;
-      n_it = (unsigned long long)P * o.n_chunks;
-      irtps::ReduceObj &q = red[r];
+      n_it = (unsigned long long)P * o.n_chunks * (b.shared ? 1 : c.K);
+      irtps::ReduceObj q;
       q.part = c.shared_part;
       q.out = c.lbar;
       q.n_chunks = o.n_chunks;
       q.n_pix = P;
       q.kc = c.K * c.C;
       q.C = c.C;
+      q.spp = spp[i];
       q.inv_spp = 1.0 / (double)spp[i];
       q.blk_begin = rblk;
       q.nblk = (int)std::min<long long>(4096, std::max<long long>(1, ((long long)P * q.kc + 2047) / 2048));
       rblk += q.nblk;
+      red.push_back(q);
     }
     begin += (unsigned)n_it;
     items += n_it;
@@ -201,15 +205,15 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
   b.primary_per_iter = primary;
   BCK(cudaMemcpyAsync(b.d_trace, h.data(), sizeof(irtps::ObjTrace) * b.n, cudaMemcpyHostToDevice, b.stream),
       "trace descriptors");
-  if (b.shared) {
-    BCK(cudaMemcpyAsync(b.d_reduce, red.data(), sizeof(irtps::ReduceObj) * b.n, cudaMemcpyHostToDevice, b.stream),
+  if (!red.empty())
+    BCK(cudaMemcpyAsync(b.d_reduce, red.data(), sizeof(irtps::ReduceObj) * red.size(), cudaMemcpyHostToDevice, b.stream),
         "partial-sum descriptors");
-    if (rblk != b.reduce_blocks && b.graph) {
-      cudaGraphExecDestroy(b.graph);
-      b.graph = nullptr;
-    }
-    b.reduce_blocks = rblk;
+  if ((rblk != b.reduce_blocks || (int)red.size() != b.n_reduce) && b.graph) {
+    cudaGraphExecDestroy(b.graph);
+    b.graph = nullptr;
   }
+  b.reduce_blocks = rblk;
+  b.n_reduce = (int)red.size();
   return IRTPS_OK;
 }
 
@@ -221,7 +225,10 @@ int enqueue_trace(irtps_batch &b, uint32_t iter, bool captured, bool timed) {
   BCK(irtps::launch_trace_batch(b.stream, b.C, b.shared, b.d_trace, b.n, b.n_items, b.d_stats[b.n].counts,
                                 b.next_item, captured ? b.iter_dev : nullptr, iter, trace_grid(b)),
       "trace launch");
-  if (b.shared) BCK(irtps::launch_parts_batch(b.stream, false, b.d_reduce, b.n, b.reduce_blocks), "partial sums");
+  if (b.shared)
+    BCK(irtps::launch_parts_batch(b.stream, false, b.d_reduce, b.n, b.reduce_blocks), "partial sums");
+  else if (b.n_reduce > 0)
+    BCK(irtps::launch_reduce_split_batch(b.stream, b.d_reduce, b.n_reduce, b.reduce_blocks), "partial sums");
   BSTAGE(ST_TRACE, false);
   return IRTPS_OK;
 }
@@ -558,7 +565,7 @@ int irtps_batch_iterate(irtps_batch *x, int n_iter, const int *spp, const int *b
   }
   rc = end_call(b, true, n_iter, out_dH);
   {  // kernels per iteration: pyramid levels, trace, PS, the solve's, two of D_H (+ counter)
-    int k = 1 + 1 + solve_kernels(b) + 2 + (b.use_graph ? 1 : 0) + (b.shared ? 2 : 0) + (b.hz_blocks > 0 ? 1 : 0) +
+    int k = 1 + 1 + solve_kernels(b) + 2 + (b.use_graph ? 1 : 0) + (b.shared ? 2 : b.n_reduce > 0 ? 1 : 0) + (b.hz_blocks > 0 ? 1 : 0) +
             irls_kernels(b);
     k += b.pyr_levels > irtps::kPyrTileLevels ? 2 : 1;
     b.stats.launches += (unsigned long long)k * n_iter;

@@ -175,14 +175,15 @@ bool trace_args_ok(Ctx &c, int spp, int bounces) {
   return true;
 }
 
-// Light-shared traces keep per-chunk partial sums; size them before any capture.
+// Light-shared traces, and per-light traces of small objects, keep per-chunk partial sums; size them before any capture.
 int prepare_trace(Ctx &c, int n_pix, int spp) {
-  if (c.opt.sampling != 1) return IRTPS_OK;
+  const size_t need = irtps::trace_scratch_floats(c, n_pix, spp);
+  if (need == 0) return IRTPS_OK;
   bool grown = false;
-  const cudaError_t e = irtps::ensure_shared_scratch(c, irtps::shared_scratch_floats(c, n_pix, spp), grown);
+  const cudaError_t e = irtps::ensure_shared_scratch(c, need, grown);
   if (e != cudaSuccess)
     return fail(c, e == cudaErrorMemoryAllocation ? IRTPS_ENOMEM : IRTPS_ECUDA,
-                std::string("light-shared partial sums: ") + cudaGetErrorString(e));
+                std::string("trace partial sums: ") + cudaGetErrorString(e));
   return IRTPS_OK;
 }
 
@@ -664,7 +665,8 @@ int irtps_render(irtps_ctx *ctx, int spp, int bounces, uint64_t seed, float sigm
   // the synthetic images take the per-light trace whatever the context's sampling
   const int sampling = c.opt.sampling;
   c.opt.sampling = 0;
-  int rc = begin_call(c);
+  int rc = prepare_trace(c, c.H * c.W, spp);
+  if (rc == IRTPS_OK) rc = begin_call(c);
   if (rc == IRTPS_OK) rc = trace_into(c, nullptr, c.H * c.W, spp, bounces, seed, 0xFFFFFFFFu, 1u, c.lbar, nullptr);
   if (rc == IRTPS_OK) rc = end_call(c, false);
   c.opt.sampling = sampling;

@@ -297,13 +297,13 @@ struct Walker {
   float bt;
   int btri;
   int flags;  // bit 0: any-hit; bits 1, 2: a second walk in x, in y; bits 3-4: current walk index; 5-6: see
-              // walker_leaf_step
+              // walker_leaf_step; 7, 8: sign bits of the direction's x and y
 };
 
-// The true direction.
+// The true direction (signs of zeros too).
 __device__ __forceinline__ F3 walker_dir(const Walker &m) {
-  return {__int_as_float(__float_as_int(m.dx) ^ (m.mx & (int)0x80000000)),
-          __int_as_float(__float_as_int(m.dy) ^ (m.my & (int)0x80000000)), m.dz};
+  return {__int_as_float(__float_as_int(m.dx) | ((m.flags << 24) & (int)0x80000000)),
+          __int_as_float(__float_as_int(m.dy) | ((m.flags << 23) & (int)0x80000000)), m.dz};
 }
 
 // (float)(n + 1) of a node index |n| < 2^22 by a magic addition (no conversion unit).
@@ -355,7 +355,8 @@ __device__ __forceinline__ bool walker_init(Walker &m, const Field &f, const Lev
   m.ax = __frcp_rn(m.dx);
   m.ay = __frcp_rn(m.dy);
   const bool on_x = floorf(o.x) == o.x, on_y = floorf(o.y) == o.y;
-  m.flags = (any ? 1 : 0) | ((on_x && d.x == 0.0f) ? 2 : 0) | ((on_y && d.y == 0.0f) ? 4 : 0);
+  m.flags = (any ? 1 : 0) | ((on_x && d.x == 0.0f) ? 2 : 0) | ((on_y && d.y == 0.0f) ? 4 : 0) |
+            (int)(((__float_as_uint(d.x) >> 31) << 7) | ((__float_as_uint(d.y) >> 31) << 8));
   m.bt = __int_as_float(0x7f800000);
   m.btri = -1;
   // a rising ray is above every vertex (by the margin) beyond this parameter; any rounding of it

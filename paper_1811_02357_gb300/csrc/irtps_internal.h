@@ -54,11 +54,12 @@ struct ObjTrace {
   uint2 key;              // Philox key {seed_lo ^ object, seed_hi}
   int EH, EW, K, spp, bounces, n_pix, shadow;
   float eps, Wf;          // ray-origin lift; W (grid units per world unit in x and y)
-  float inv_w2;           // 1 / W^2
+  float inv_w;            // 1 / W, rounded to nearest
   unsigned item_begin;    // first work item of the object (batched launches)
   uint32_t iter0;         // added to the launch's iteration field
-  float *part;            // light-shared sampling: partial sums, n_chunks x n_pix x K x C, then n_chunks x n_pix x C
-  int n_chunks, chunk;    // light-shared sampling: sample chunks per pixel and samples per chunk
+  float *part;            // partial sums; light-shared sampling: n_chunks x n_pix x K x C, then n_chunks x n_pix x C;
+                          // per light with n_chunks > 1: the samples' radiances, spp x K x C x n_pix
+  int n_chunks, chunk;    // sample chunks per pixel (light-shared) or (pixel, light), samples per chunk
   const float *hz;        // horizon bounds, 8 octants x H W (null: no early escape)
   uint8_t *hole;          // per-light sampling: K x n_pix, 1 where no sample's first segment hit (null: none)
   int hz_stride;          // H W
@@ -291,7 +292,7 @@ cudaError_t launch_render(Ctx &c, uint64_t seed, float sigma, const float *lbar,
 // resident blocks of the (batched) trace kernel, per-light or light-shared, 0 if unknown
 int trace_grid_limit(int C, int n_obj = 0, bool shared = false);
 void fill_obj_trace(const Ctx &c, ObjTrace &o);  // descriptor of a context's object (no sampling fields)
-size_t shared_scratch_floats(const Ctx &c, int n_pix, int spp);  // light-shared chunk partials needed
+size_t trace_scratch_floats(const Ctx &c, int n_pix, int spp);  // chunk partials a trace needs (0: none)
 cudaError_t launch_trace_batch(cudaStream_t s, int C, bool shared, const ObjTrace *d_objs, int n_obj,
                                unsigned n_items, unsigned long long *counts, unsigned *next_item,
                                const uint32_t *iter_dev, uint32_t iter, int grid_limit);
@@ -300,14 +301,16 @@ struct SharedSplit {
   int n_chunks, chunk;  // as in ObjTrace
 };
 SharedSplit shared_split(int n_pix, int spp);
+SharedSplit light_split(const Ctx &c, int spp);  // per-light sampling (one chunk unless the object is small)
 cudaError_t ensure_shared_scratch(Ctx &c, size_t need, bool &grown);
 struct ReduceObj {
-  float *part;     // n_chunks x n_pix x kc light partial sums, then n_chunks x n_pix x C environment sums
+  float *part;     // as in ObjTrace
   float *out;      // kc x n_pix (Lbar)
-  int n_chunks, n_pix, kc, C;
+  int n_chunks, n_pix, kc, C, spp;
   double inv_spp;
   int blk_begin, nblk;
 };
+cudaError_t launch_reduce_split_batch(cudaStream_t s, const ReduceObj *d_objs, int n, int blocks);
 cudaError_t launch_parts_batch(cudaStream_t s, bool zero, const ReduceObj *d_objs, int n, int blocks);
 cudaError_t launch_probe_dirs(cudaStream_t s, int n, const float *normals, const uint32_t *x0, const uint32_t *x1,
                               float *out);
