@@ -47,7 +47,7 @@ void release(Ctx &c) {
                   c.cg_x, c.cg_b, c.cg_r, c.cg_z, c.cg_p, c.cg_ap, c.part, c.dstats, c.next_item, c.cg_ctl,
                   c.mg_x0, c.mg_x1, c.mg_b, c.mg_wh, c.mg_wv, c.mg_wh_unit, c.mg_wv_unit, c.iter_dev, c.holes,
                   c.fill_v, c.fill_w, c.sp_pool, c.sp_t, c.ps_pix, c.ps_mask,
-                  c.ps_rhs, c.ps_count};
+                  c.ps_rhs, c.ps_count, c.ps_mtab};
   for (void *b : bufs)
     if (b) cudaFree(b);
   if (c.h_part) cudaFreeHost(c.h_part);
@@ -413,6 +413,7 @@ int irtps_create(irtps_ctx **out, int H, int W, int K, int C, const float *light
       (rc = dalloc(c, &c.ps_pix, P, "masked-pixel list")) || (rc = dalloc(c, &c.ps_mask, P, "masked-pixel list")) ||
       (rc = dalloc(c, &c.ps_rhs, (size_t)9 * P, "masked-pixel list")) ||
       (rc = dalloc(c, &c.ps_count, 1, "masked-pixel list")) ||
+      (rc = dalloc(c, &c.ps_mtab, (size_t)6 * K, "light products")) ||
       (rc = dalloc(c, &c.pmax, (size_t)total, "pyramid")) || (rc = dalloc(c, &c.planes, (size_t)total, "pyramid")) ||
       (rc = dalloc(c, &c.cg_x, P, "cg")) || (rc = dalloc(c, &c.cg_b, P, "cg")) ||
       (rc = dalloc(c, &c.cg_r, P, "cg")) || (rc = dalloc(c, &c.cg_z, P, "cg")) ||
@@ -471,6 +472,11 @@ int irtps_create(irtps_ctx **out, int H, int W, int K, int C, const float *light
                       cudaMemcpyHostToDevice, c.stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(c.d_lights, c.h_lights.data(), sizeof(float) * K * 3, cudaMemcpyHostToDevice, c.stream);
+  std::vector<long long> products;
+  irtps::ps_light_products(c.h_lights.data(), K, products, c.ps_mscale);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(c.ps_mtab, products.data(), sizeof(long long) * products.size(), cudaMemcpyHostToDevice,
+                        c.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.lbar, 0, sizeof(float) * K * C * P, c.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.depth, 0, sizeof(float) * P, c.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.albedo, 0, sizeof(float) * C * P, c.stream);

@@ -156,6 +156,8 @@ struct Ctx {
   unsigned long long *ps_mask = nullptr;  // right-hand sides (9 floats each), count
   float *ps_rhs = nullptr;
   unsigned *ps_count = nullptr;
+  long long *ps_mtab = nullptr;   // PS: fixed-point products of the lights, 6 per light (ps_light_products)
+  double ps_mscale = 0.0;
   float *pmax = nullptr;          // pyramid of maxima, all levels
   uint2 *planes = nullptr;        // bounding planes of the same nodes
   int levels = 0;
@@ -319,6 +321,7 @@ cudaError_t launch_probe_rays(Ctx &c, int n, const float *rays, float *t_out, in
 // pixels per thread the PS kernel takes: the tuned width when the pixel count is a multiple of it, else 1
 inline int ps_vec_for(const Ctx &c) { return (c.H * c.W) % c.ps_vec == 0 ? c.ps_vec : 1; }
 cudaError_t launch_ps(Ctx &c, bool zero_indirect);
+void ps_light_products(const float *lights, int K, std::vector<long long> &tab, double &scale);
 size_t ps_args_bytes();
 void ps_fill_args(const Ctx &c, bool zero_indirect, int blk_begin, void *dst);
 cudaError_t launch_ps_batch(cudaStream_t s, int C, int dtype, const void *d_args, int n, int blocks);

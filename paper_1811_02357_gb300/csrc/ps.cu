@@ -2,7 +2,7 @@
 //
 // Per pixel p: I(k, c) = A0(k, c, p) - rho_t(c, p) * Lbar(k, c, p); row k is valid
 // iff tau_lo < mean_c I(k, c) < tau_hi (decided in FP32, each operation rounded
-// on its own).  All rows valid: G_c = pinv(L) I_c with pinv(L) = (L^T L)^-1 L^T
+// on its own; the division by 3 moved into the bounds, channel_sum_bounds).  All rows valid: G_c = pinv(L) I_c with pinv(L) = (L^T L)^-1 L^T
 // (Eq. 4), summed as pinv(L) I, or - when L^T L is well conditioned (1-norm
 // condition number at most 16, decided on the host in FP64) - as (L^T L)^-1 (L^T I),
 // the same product associated the other way, which needs only the one running
@@ -15,8 +15,11 @@
 // 6*K*C flops: far below the tensor-core ridge, so it runs on the FP32 pipes
 // with coalesced [k][c][p] loads and the pixel's state written once.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <limits>
+#include <vector>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -31,7 +34,9 @@ struct PSArgs {
   float4 *nrm;
   uint8_t *valid;
   int P, K;
-  float tau_lo, tau_hi;
+  float sum_lo, sum_hi; // row k is valid iff sum_lo < sum_c I(k, c) < sum_hi (see channel_sum_bounds)
+  const longlong2 *mtab;  // per light the six products l_u l_v in fixed point (3 x longlong2)
+  double mscale;          // value of one unit of mtab
   double cond_max;
   int zero_indirect;    // 1: Lbar taken as 0 (iteration 0, classic PS)
   float pinv[3][kMaxLights];
@@ -59,9 +64,8 @@ __device__ __forceinline__ void ps_row(const PSArgs &a, int k, const float *rho,
   float I[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) I[c] = __fsub_rn(a0[c], __fmul_rn(rho[c], lb[c]));
-  float chat = I[0];
-  if (C == 3) chat = __fdiv_rn(__fadd_rn(__fadd_rn(I[0], I[1]), I[2]), 3.0f);
-  const bool ok = chat > a.tau_lo && chat < a.tau_hi;
+  const float sum = C == 3 ? __fadd_rn(__fadd_rn(I[0], I[1]), I[2]) : I[0];
+  const bool ok = sum > a.sum_lo && sum < a.sum_hi;
   if (ok) valid |= 1ull << k;
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
@@ -87,9 +91,18 @@ __device__ __forceinline__ void ps_apply_minv(const PSArgs &a, const float (&R)[
   }
 }
 
+// |(x, y, z)| with the fused multiply-adds written out, so that its bits do not depend on the code around it (a
+// last-bit change of an estimate can send a later iteration's ray past an edge): z last, y or x before it.
+__device__ __forceinline__ float norm_zyx(float x, float y, float z) {
+  return sqrtf(__fmaf_rn(z, z, __fmaf_rn(y, y, __fmul_rn(x, x))));
+}
+__device__ __forceinline__ float norm_zxy(float x, float y, float z) {
+  return sqrtf(__fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y))));
+}
+
 // Normal and albedo of pixel p from G (Eq. 4 and the text after it): n = normalize(sum_c G_c),
 // rho_c = |G_c|; a pixel whose solve failed (ok false) or whose sum vanishes is invalid.
-template <int C>
+template <int C, bool LISTED = false>
 __device__ __forceinline__ void ps_store(const PSArgs &a, int p, const float (&G)[3][C], bool ok) {
   const size_t P = (size_t)a.P;
   float sx = 0.0f, sy = 0.0f, sz = 0.0f;
@@ -99,14 +112,14 @@ __device__ __forceinline__ void ps_store(const PSArgs &a, int p, const float (&G
     sy += G[1][c];
     sz += G[2][c];
   }
-  const float norm = sqrtf(sx * sx + sy * sy + sz * sz);
+  const float norm = norm_zyx(sx, sy, sz);
   if (!(norm > 0.0f) || !isfinite(norm)) ok = false;
   float4 out = make_float4(0.0f, 0.0f, 1.0f, 0.0f);
   float rsum = 0.0f;
   float rout[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    rout[c] = ok ? sqrtf(G[0][c] * G[0][c] + G[1][c] * G[1][c] + G[2][c] * G[2][c]) : 0.0f;
+    rout[c] = !ok ? 0.0f : (C == 1 && LISTED) ? norm : norm_zxy(G[0][c], G[1][c], G[2][c]);
     rsum += rout[c];
   }
   if (ok) {
@@ -122,11 +135,11 @@ __device__ __forceinline__ void ps_store(const PSArgs &a, int p, const float (&G
 // A pixel with masked rows: the normal equations (L_v^T L_v) G_c = L_v^T I_v,c over the
 // valid rows, R = L_v^T I the FP32 sum of ps_row.  A well-conditioned system (FP32
 // condition number at most kRefineCond, the common case) is solved in FP32.  Otherwise
-// the matrix is summed from the lights in double-float arithmetic and its inverse (by the
+// the matrix is summed from the lights in fixed point and its inverse (by the
 // adjugate) and 1-norm condition number are formed in FP64; fewer than 3 rows, a singular
 // or ill-conditioned system (condition above cond_max): ok = false; and R, whose FP32
-// rounding the condition number would amplify, is summed again in double-float from the
-// pixel's valid rows (read again).
+// rounding the condition number would amplify, is summed again in twice the precision from
+// the pixel's valid rows (read again).
 constexpr double kRefineCond = 16.0;
 enum : int { PS_SOLVED = 0, PS_INVALID = 1, PS_NEED_FP64 = 2 };
 
@@ -175,15 +188,16 @@ __device__ __forceinline__ int ps_masked_fp32(const PSArgs &a, const float (&R)[
   return PS_NEED_FP64;
 }
 
-// The part that FP32 passed on (ps_masked_fp32): the matrix L_v^T L_v and the right-hand side
-// in double-float arithmetic, the inverse (by the adjugate) and the 1-norm condition number in
-// FP64; singular or above cond_max: false.  Above kRefineCond the right-hand side is summed again
-// from the pixel's valid rows (read again), since the condition number would amplify the FP32
-// rounding of the streaming pass's sum.  GB300's FP64 pipe is narrow, so the sums, which are
-// most of the work, run on the FP32 pipes as double-float values (hi + lo, about 48 bits), built
-// from error-free transformations: Knuth's two-sum and the fused-multiply-add two-product.
-// Every operation is rounded on its own (the _rn intrinsics keep the compiler from fusing or
-// reordering them), so the per-thread uses of these helpers give the same bits everywhere.
+// The part that FP32 passed on (ps_masked_fp32): the matrix L_v^T L_v, its inverse (by the adjugate) and the 1-norm
+// condition number in FP64; singular or above cond_max: false.  Above kRefineCond the right-hand side is summed again
+// from the pixel's valid rows (read again), since the condition number would amplify the FP32 rounding of the
+// streaming pass's sum.  GB300's FP64 pipe is narrow, so the sums, which are most of the work, stay off it:
+//  - the matrix as 64-bit integer sums of the lights' fixed-point products (ps_light_products): two integer
+//    additions a term instead of a double-float product and addition (about 25 operations);
+//  - the right-hand side by compensated FP32 sums (Ogita, Rump and Oishi's dot product in twice the working
+//    precision, about 48 bits): error-free two-sum and fused-multiply-add two-product, the errors summed beside.
+// Every operation is rounded on its own (the _rn intrinsics keep the compiler from fusing or reordering them), so the
+// per-thread uses of these helpers give the same bits everywhere.
 struct DF {
   float hi, lo;
 };
@@ -192,37 +206,11 @@ __device__ __forceinline__ DF df_two_sum(float a, float b) {
   const float bb = __fsub_rn(s, a);
   return DF{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
 }
-__device__ __forceinline__ DF df_fast_two_sum(float a, float b) {  // needs |a| >= |b| (or a = 0)
-  const float s = __fadd_rn(a, b);
-  return DF{s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ DF df_add(DF x, DF y) {
-  const DF s = df_two_sum(x.hi, y.hi);
-  const DF t = df_two_sum(x.lo, y.lo);
-  const DF u = df_fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
-  return df_fast_two_sum(u.hi, __fadd_rn(u.lo, t.lo));
-}
 // x * b exactly as hi + lo (two-product)
 __device__ __forceinline__ DF df_prod(float x, float b) {
   const float p = __fmul_rn(x, b);
   return DF{p, __fmaf_rn(x, b, -p)};
 }
-__device__ __forceinline__ DF df_mul_f(DF x, float b) {
-  const DF p = df_prod(x.hi, b);
-  return df_fast_two_sum(p.hi, __fmaf_rn(x.lo, b, p.lo));
-}
-__device__ __forceinline__ double df_to_double(DF x) { return (double)x.hi + (double)x.lo; }
-
-// Entry (u, v) of L_v^T L_v, over the valid rows in light order (each product exact).
-__device__ __forceinline__ double ps_m_df(const PSArgs &a, unsigned long long valid, int u, int v) {
-  DF s = {0.0f, 0.0f};
-  for (int k = 0; k < a.K; ++k)
-    if ((valid >> k) & 1ull) s = df_add(s, df_prod(a.light[k][u], a.light[k][v]));
-  return df_to_double(s);
-}
-// the six entries m00 m01 m02 m11 m12 m22
-__device__ __constant__ const int kMu[6] = {0, 0, 0, 1, 1, 2};
-__device__ __constant__ const int kMv[6] = {0, 1, 2, 1, 2, 2};
 
 // Inverse (m00 m01 m02 m11 m12 m22 layout) and 1-norm condition number; false when the
 // system is singular or above cond_max.
@@ -247,48 +235,133 @@ __device__ __forceinline__ bool ps_inv64(const PSArgs &a, const double (&M)[6], 
   return cond <= a.cond_max;
 }
 
+// R = L_v^T I of pixel p's valid rows in twice the working precision (hi + lo).
 template <int C, typename TI>
-__device__ __forceinline__ bool ps_masked_fp64(const PSArgs &a, int p, const float (&R)[3][C], float (&G)[3][C],
-                                               unsigned long long valid) {
-  double M[6], I[6], cond;
+__device__ __forceinline__ void ps_rhs_twofold(const PSArgs &a, int p, unsigned long long valid, float (&hi)[3][C],
+                                               float (&lo)[3][C]) {
+  const TI *img = reinterpret_cast<const TI *>(a.images);
+  const size_t P = (size_t)a.P;
+  float rho[C];
 #pragma unroll
-  for (int e = 0; e < 6; ++e) M[e] = ps_m_df(a, valid, kMu[e], kMv[e]);
-  if (!ps_inv64(a, M, I, cond)) return false;
-  double Rd[3][C];
+  for (int c = 0; c < C; ++c) rho[c] = a.zero_indirect ? 0.0f : a.albedo[c * P + p];
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
-    for (int c = 0; c < C; ++c) Rd[r][c] = R[r][c];
-  if (cond > kRefineCond) {  // ill-conditioned: the right-hand side again, in double-float
-    const TI *img = reinterpret_cast<const TI *>(a.images);
-    const size_t P = (size_t)a.P;
-    float rho[C];
+    for (int c = 0; c < C; ++c) hi[r][c] = lo[r][c] = 0.0f;
+#pragma unroll 2
+  for (int k = 0; k < a.K; ++k) {
+    if (!((valid >> k) & 1ull)) continue;
 #pragma unroll
-    for (int c = 0; c < C; ++c) rho[c] = a.zero_indirect ? 0.0f : a.albedo[c * P + p];
-    DF Rf[3][C];
+    for (int c = 0; c < C; ++c) {
+      const size_t o = ((size_t)k * C + c) * P + p;
+      const float a0 = load_img<TI>(img + o);
+      const float lb = a.zero_indirect ? 0.0f : __ldg(a.lbar + o);
+      // I = a0 - rho lb = d.hi + (d.lo - q.lo): rho lb = q.hi + q.lo exactly
+      const DF q = df_prod(rho[c], lb);
+      const DF d = df_two_sum(a0, -q.hi);
+      const float il = __fsub_rn(d.lo, q.lo);
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int c = 0; c < C; ++c) Rf[r][c] = DF{0.0f, 0.0f};
-    for (int k = 0; k < a.K; ++k) {
-      if (!((valid >> k) & 1ull)) continue;
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const size_t o = ((size_t)k * C + c) * P + p;
-        const float a0 = load_img<TI>(img + o);
-        const float lb = a.zero_indirect ? 0.0f : __ldg(a.lbar + o);
-        // I = a0 - rho lb: rho lb = q.hi + q.lo exactly, then two exact-error subtractions
-        const DF q = df_prod(rho[c], lb);
-        const DF d = df_two_sum(a0, -q.hi);
-        const DF iv = df_two_sum(d.hi, __fsub_rn(d.lo, q.lo));
-#pragma unroll
-        for (int r = 0; r < 3; ++r) Rf[r][c] = df_add(Rf[r][c], df_mul_f(iv, a.light[k][r]));
+      for (int r = 0; r < 3; ++r) {
+        const float l = a.light[k][r];
+        const DF t = df_prod(l, d.hi);
+        const DF s = df_two_sum(hi[r][c], t.hi);
+        hi[r][c] = s.hi;
+        lo[r][c] = __fadd_rn(__fmaf_rn(l, il, lo[r][c]), __fadd_rn(s.lo, t.lo));
       }
     }
+  }
+}
+
+// Systems of a condition number up to kTwofoldCond are solved in FP32 and refined twice: G = M^-1 R from the FP32
+// inverse, then G += M^-1 (R - M G), the residual in twice the precision (M as hi + lo).  The error of the first G,
+// about 4 * 2^-24 cond relative (1.2e-4 at 512), is squared by the first step; the second one's correction is about
+// an ulp of G, known to 1e-4 of itself, so that G is the exact solution's rounding but for one pixel in ten
+// thousand or fewer.  Such a system is certainly below cond_max.  Beyond it the inverse and the products are FP64, whose 130 or so
+// operations a pixel bound this kernel (16 cycles of the SM's FP64 pipe per warp instruction).
+constexpr double kTwofoldCond = 512.0;
+
+template <int C, typename TI>
+__device__ __forceinline__ bool ps_masked_fp64(const PSArgs &a, int p, const float (&R)[3][C], float (&G)[3][C],
+                                               unsigned long long valid) {
+  long long m[6] = {0, 0, 0, 0, 0, 0};
+  for (int k = 0; k < a.K; ++k) {
+    const longlong2 p2 = __ldg(a.mtab + 3 * k), q2 = __ldg(a.mtab + 3 * k + 1), r2 = __ldg(a.mtab + 3 * k + 2);
+    if (!((valid >> k) & 1ull)) continue;
+    m[0] += p2.x;
+    m[1] += p2.y;
+    m[2] += q2.x;
+    m[3] += q2.y;
+    m[4] += r2.x;
+    m[5] += r2.y;
+  }
+  const float sc = (float)a.mscale;
+  if (kTwofoldCond <= 0.5 * a.cond_max && sc > 1e-30f && sc < 1e10f) {
+    float mh[6], ml[6];
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+      mh[e] = __ll2float_rn(m[e]);
+      ml[e] = __ll2float_rn(m[e] - __float2ll_rn(mh[e])) * sc;
+      mh[e] *= sc;
+    }
+    const float a00 = mh[3] * mh[5] - mh[4] * mh[4], a01 = mh[2] * mh[4] - mh[1] * mh[5],
+                a02 = mh[1] * mh[4] - mh[2] * mh[3], a11 = mh[0] * mh[5] - mh[2] * mh[2],
+                a12 = mh[1] * mh[2] - mh[0] * mh[4], a22 = mh[0] * mh[3] - mh[1] * mh[1];
+    const float det = mh[0] * a00 + mh[1] * a01 + mh[2] * a02;
+    const float nm = fmaxf(fabsf(mh[0]) + fabsf(mh[1]) + fabsf(mh[2]),
+                           fmaxf(fabsf(mh[1]) + fabsf(mh[3]) + fabsf(mh[4]), fabsf(mh[2]) + fabsf(mh[4]) + fabsf(mh[5])));
+    const float na = fmaxf(fabsf(a00) + fabsf(a01) + fabsf(a02),
+                           fmaxf(fabsf(a01) + fabsf(a11) + fabsf(a12), fabsf(a02) + fabsf(a12) + fabsf(a22)));
+    if (det > 0.0f && isfinite(det) && nm * na <= (float)kTwofoldCond * det) {
+      float hi[3][C], lo[3][C];
+      ps_rhs_twofold<C, TI>(a, p, valid, hi, lo);
+      const float id = 1.0f / det;
+      const float iv[3][3] = {{a00 * id, a01 * id, a02 * id}, {a01 * id, a11 * id, a12 * id}, {a02 * id, a12 * id, a22 * id}};
+      constexpr int ix[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        float g[3], res[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) g[u] = iv[u][0] * hi[0][c] + iv[u][1] * hi[1][c] + iv[u][2] * hi[2][c];
+#pragma unroll 1
+        for (int step = 0; step < 2; ++step) {
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            float h = hi[u][c], l = lo[u][c];
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+              const DF t = df_prod(-mh[ix[u][v]], g[v]);
+              const DF s = df_two_sum(h, t.hi);
+              h = s.hi;
+              l = __fadd_rn(__fmaf_rn(-ml[ix[u][v]], g[v], l), __fadd_rn(s.lo, t.lo));
+            }
+            res[u] = h + l;
+          }
+#pragma unroll
+          for (int u = 0; u < 3; ++u) g[u] += iv[u][0] * res[0] + iv[u][1] * res[1] + iv[u][2] * res[2];
+        }
+#pragma unroll
+        for (int u = 0; u < 3; ++u) G[u][c] = g[u];
+      }
+      return true;
+    }
+  }
+  double M[6], I[6], cond;
+#pragma unroll
+  for (int e = 0; e < 6; ++e) M[e] = (double)m[e] * a.mscale;
+  if (!ps_inv64(a, M, I, cond)) return false;
+  double Rd[3][C];
+  if (cond > kRefineCond) {  // ill-conditioned: the right-hand side again, in twice the precision
+    float hi[3][C], lo[3][C];
+    ps_rhs_twofold<C, TI>(a, p, valid, hi, lo);
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
-      for (int c = 0; c < C; ++c) Rd[r][c] = df_to_double(Rf[r][c]);
+      for (int c = 0; c < C; ++c) Rd[r][c] = (double)hi[r][c] + (double)lo[r][c];
+  } else {
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int c = 0; c < C; ++c) Rd[r][c] = R[r][c];
   }
 #pragma unroll
   for (int c = 0; c < C; ++c) {
@@ -428,11 +501,15 @@ struct PSList {
 #endif
 // resident blocks per SM asked of the normal-equation form (its state fits 64 registers at V <= 2)
 constexpr int kPsMinBlocks = IRTPS_PS_MINB;
+#ifndef IRTPS_PS_MINB1
+#define IRTPS_PS_MINB1 5
+#endif
+constexpr int kPsMinBlocks1 = IRTPS_PS_MINB1;  // one pixel a thread needs fewer registers
 // lights per unrolled step of the streaming loop, over all V pixels of a thread
 constexpr int kPsKUnroll = IRTPS_PS_KUNROLL;
 
 template <int C, typename TI, int V, bool NE>
-__global__ void __launch_bounds__(256, (NE && V < 4) ? kPsMinBlocks : 2) k_ps_fast(const PSArgs a, const PSList L) {
+__global__ void __launch_bounds__(256, (NE && V < 4) ? (V == 1 ? kPsMinBlocks1 : kPsMinBlocks) : 2) k_ps_fast(const PSArgs a, const PSList L) {
   const int p = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   const bool in = p < a.P;
   const TI *img = reinterpret_cast<const TI *>(a.images);
@@ -520,8 +597,12 @@ __global__ void __launch_bounds__(256, (NE && V < 4) ? kPsMinBlocks : 2) k_ps_fa
 
 // The listed pixels, one per thread (the FP64 pipe is narrow: a pixel's FP64 work stays in
 // one lane), a grid-stride loop over the list.
+#ifndef IRTPS_PS_MASKED_BLOCKS
+#define IRTPS_PS_MASKED_BLOCKS 8
+#endif
+constexpr int kPsMaskedBlocks = IRTPS_PS_MASKED_BLOCKS;  // resident blocks per SM (its loads' latency bounds it)
 template <int C, typename TI>
-__global__ void __launch_bounds__(128) k_ps_masked(const PSArgs a, const PSList L) {
+__global__ void __launch_bounds__(128, kPsMaskedBlocks) k_ps_masked(const PSArgs a, const PSList L) {
   const unsigned n = *L.count;
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int p = L.pix[i];
@@ -531,7 +612,7 @@ __global__ void __launch_bounds__(128) k_ps_masked(const PSArgs a, const PSList 
 #pragma unroll
       for (int c = 0; c < C; ++c) R[r][c] = L.rhs[(size_t)i * 9 + r * C + c];
     const bool ok = ps_masked_fp64<C, TI>(a, p, R, G, L.mask[i]);
-    ps_store<C>(a, p, G, ok);
+    ps_store<C, true>(a, p, G, ok);
   }
 }
 
@@ -708,9 +789,8 @@ __global__ void __launch_bounds__(kTcRows) k_ps_tc(const PSArgs a, unsigned long
 #pragma unroll
       for (int e = 0; e < CH; e += C) {
         const int k = (q0 + e) / C;
-        float chat = I[e];
-        if (C == 3) chat = __fdiv_rn(__fadd_rn(__fadd_rn(I[e], I[e + 1]), I[e + 2]), 3.0f);
-        const bool ok = q0 + e < kc && chat > a.tau_lo && chat < a.tau_hi;
+        const float sum = C == 3 ? __fadd_rn(__fadd_rn(I[e], I[e + 1]), I[e + 2]) : I[e];
+        const bool ok = q0 + e < kc && sum > a.sum_lo && sum < a.sum_hi;
         if (ok) valid |= 1ull << k;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
@@ -780,6 +860,48 @@ __global__ void __launch_bounds__(kTcRows) k_ps_tc(const PSArgs a, unsigned long
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
 }
 
+// Bounds on the sum of the channels: the FP32 quotient sum / 3 is monotone in the sum, so "quotient > tau_lo" is
+// "sum > the largest sum whose quotient is not", and "< tau_hi" likewise: the same decisions without a division
+// per row (found here by stepping from 3 tau).
+static void channel_sum_bounds(int C, float tau_lo, float tau_hi, float &lo, float &hi) {
+  lo = tau_lo;
+  hi = tau_hi;
+  if (C == 1) return;
+  auto q = [](float x) { return (float)(x / 3.0f); };
+  if (std::isfinite(tau_lo)) {
+    float x = 3.0f * tau_lo;
+    if (std::isinf(x)) x = std::copysign(std::numeric_limits<float>::max(), x);
+    while (q(x) > tau_lo) x = std::nextafter(x, -INFINITY);
+    while (q(std::nextafter(x, INFINITY)) <= tau_lo) x = std::nextafter(x, INFINITY);
+    lo = x;
+  }
+  if (std::isfinite(tau_hi)) {
+    float x = 3.0f * tau_hi;
+    if (std::isinf(x)) x = std::copysign(std::numeric_limits<float>::max(), x);
+    while (q(x) < tau_hi) x = std::nextafter(x, INFINITY);
+    while (q(std::nextafter(x, -INFINITY)) >= tau_hi) x = std::nextafter(x, -INFINITY);
+    hi = x;
+  }
+}
+
+// Fixed-point table of the lights' products l_u l_v (00 01 02 11 12 22): units of 2^-s, s such that the sum over all
+// lights fits 62 bits.  The products of two FP32 numbers are exact in FP64, the table's rounding is 2^-56 of the
+// largest product or less, and integer sums are exact in any order.
+void ps_light_products(const float *lights, int K, std::vector<long long> &tab, double &scale) {
+  static const int u[6] = {0, 0, 0, 1, 1, 2}, v[6] = {0, 1, 2, 1, 2, 2};
+  double big = 0.0;
+  for (int k = 0; k < K; ++k)
+    for (int e = 0; e < 6; ++e) big = std::max(big, std::fabs((double)lights[3 * k + u[e]] * lights[3 * k + v[e]]));
+  int ex = 0;
+  std::frexp(big * K, &ex);  // big K < 2^ex
+  const int s = 62 - ex;
+  tab.resize((size_t)6 * K);
+  for (int k = 0; k < K; ++k)
+    for (int e = 0; e < 6; ++e)
+      tab[(size_t)6 * k + e] = std::llrint(std::ldexp((double)lights[3 * k + u[e]] * lights[3 * k + v[e]], s));
+  scale = std::ldexp(1.0, -s);
+}
+
 static void fill_ps_args(const Ctx &c, bool zero_indirect, PSArgs &a) {
   a.images = c.images;
   a.lbar = c.lbar;
@@ -788,8 +910,9 @@ static void fill_ps_args(const Ctx &c, bool zero_indirect, PSArgs &a) {
   a.valid = c.valid;
   a.P = c.H * c.W;
   a.K = c.K;
-  a.tau_lo = c.opt.tau_lo;
-  a.tau_hi = c.opt.tau_hi;
+  channel_sum_bounds(c.C, c.opt.tau_lo, c.opt.tau_hi, a.sum_lo, a.sum_hi);
+  a.mtab = (const longlong2 *)c.ps_mtab;
+  a.mscale = c.ps_mscale;
   a.cond_max = c.opt.cond_max;
   a.zero_indirect = zero_indirect ? 1 : 0;
   for (int k = 0; k < c.K; ++k) {
@@ -874,7 +997,7 @@ static cudaError_t launch_ps_split(Ctx &c, const PSArgs &a) {
   else
     launch_ps_fast<C, TI, false>(c, a, L, v, blocks);
   // the listed pixels (few: ill-conditioned masked systems), a grid-stride loop over the list
-  const int cap = 4 * (c.sms > 0 ? c.sms : 1);
+  const int cap = kPsMaskedBlocks * (c.sms > 0 ? c.sms : 1);
   const unsigned mblocks = (unsigned)std::min<long long>(cap, ((long long)a.P + 127) / 128);
   k_ps_masked<C, TI><<<mblocks, 128, 0, c.stream>>>(a, L);
   return cudaGetLastError();
