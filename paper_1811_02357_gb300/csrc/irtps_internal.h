@@ -98,7 +98,7 @@ struct FftPlan {
 // One direct (spectral) depth solve.
 struct SpecObj {
   int H, W;
-  double h, tol;
+  double h, inv_p, tol;  // pixel pitch, 1 / (H W), tolerance
   float nz_min;
   const float4 *nrm;
   float *depth;

@@ -233,6 +233,7 @@ cudaError_t spectral_setup(Ctx &c) {
 SpecObj spec_object(const Ctx &c, CGAcc *acc) {
   SpecObj o = c.sp;
   o.h = 1.0 / (double)c.W;
+  o.inv_p = 1.0 / ((double)c.H * c.W);
   o.nz_min = c.opt.nz_min;
   o.tol = c.opt.cg_tol;
   o.nrm = c.nrm;

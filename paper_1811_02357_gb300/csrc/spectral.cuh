@@ -427,7 +427,7 @@ __device__ __forceinline__ void check(const SpecObj &o, int blk, int nblk) {
   double rr = 0.0;
   for (int i = threadIdx.x; i < o.row_blocks; i += blockDim.x) rr += __ldcg(o.part + o.row_blocks + i);
   rr = block_sum(rr, sh);
-  if (threadIdx.x == 0) s_mean = rr / (double)P;
+  if (threadIdx.x == 0) s_mean = rr * o.inv_p;
   __syncthreads();
   const double mean = s_mean;
   float rf = 0.0f;
@@ -457,9 +457,9 @@ __device__ __forceinline__ void check(const SpecObj &o, int blk, int nblk) {
   rr = block_sum(rr, sh);
   if (threadIdx.x == 0) {
     CGCtl *ctl = o.ctl;
+    // one FP64 division and a FP32 root: a chain of FP64 roots by one thread takes longer than the pass itself
     ctl->count = 0u;
-    ctl->bnorm = sqrt(bb);
-    ctl->rel = bb > 0.0 ? sqrt(rr) / sqrt(bb) : 0.0;
+    ctl->rel = bb > 0.0 ? (double)sqrtf((float)(rr / bb)) : 0.0;
     ctl->iters = 1;
     o.acc->iters += 1;
     o.acc->last_iters = 1;
