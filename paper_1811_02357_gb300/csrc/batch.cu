@@ -141,7 +141,7 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
   for (int i = 0; i < b.n; ++i) order[i] = i;
   auto cost = [&](int i) -> long long {  // samples x bounces of one work item (x K when shared)
     const Ctx &c = b.objs[i]->c;
-    if (!b.shared) return (long long)irtps::light_split(c, spp[i]).chunk * bounces[i];
+    if (!b.shared) return (long long)irtps::light_split(c, c.H * c.W, spp[i]).chunk * bounces[i];
     return (long long)irtps::shared_split(c.H * c.W, spp[i]).chunk * bounces[i] * c.K;
   };
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
@@ -151,6 +151,7 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
   unsigned long long primary = 0, items = 0;
   int rblk = 0;
   bool grown = false;
+  size_t split_left = irtps::kSplitBytes / sizeof(float);  // the split objects' radiances, all together
   for (int r = 0; r < b.n; ++r) {
     const int i = order[r];
     Ctx &c = b.objs[i]->c;
@@ -167,12 +168,26 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
     o.iter0 = c.t;
     unsigned long long n_it = (unsigned long long)P * c.K;
     // (chunk, pixel) items, or (chunk, light, pixel) items of a small object: partial sums in the object's scratch
-    const irtps::SharedSplit sp = b.shared ? irtps::shared_split(P, spp[i]) : irtps::light_split(c, spp[i]);
+    irtps::SharedSplit sp = b.shared ? irtps::shared_split(P, spp[i]) : irtps::light_split(c, P, spp[i]);
+    if (!b.shared && sp.n_chunks > 1) {  // without room an object is traced unsplit (same bits)
+      const size_t need = irtps::trace_scratch_floats(c, P, spp[i]);
+      bool g = false;
+      cudaError_t e = cudaErrorMemoryAllocation;
+      if (need <= split_left) e = irtps::ensure_shared_scratch(c, need, g);
+      grown = grown || g;
+      if (e == cudaSuccess)
+        split_left -= need;
+      else if (e == cudaErrorMemoryAllocation)
+        sp = {1, spp[i]};
+      else
+        BCK(e, "trace partial sums");
+    }
     o.n_chunks = sp.n_chunks;
     o.chunk = sp.chunk;
     if (b.shared || sp.n_chunks > 1) {
       bool g = false;
-      BCK(irtps::ensure_shared_scratch(c, irtps::trace_scratch_floats(c, P, spp[i]), g), "trace partial sums");
+      if (b.shared)
+        BCK(irtps::ensure_shared_scratch(c, irtps::trace_scratch_floats(c, P, spp[i]), g), "trace partial sums");
       grown = grown || g;
       o.part = c.shared_part;
       n_it = (unsigned long long)P * o.n_chunks * (b.shared ? 1 : c.K);
@@ -201,17 +216,17 @@ int upload_trace(irtps_batch &b, const int *spp, const int *bounces, uint64_t se
   // claims run past the last item by at most one per lane: keep the counter far from wrapping
   if (items > (1ull << 32) - (1ull << 24))
     return bfail(b, IRTPS_EINVAL, "batch: too many work items (objects x lights x pixels >= 2^32 - 2^24)");
-  b.n_items = begin;
   b.primary_per_iter = primary;
   BCK(cudaMemcpyAsync(b.d_trace, h.data(), sizeof(irtps::ObjTrace) * b.n, cudaMemcpyHostToDevice, b.stream),
       "trace descriptors");
   if (!red.empty())
     BCK(cudaMemcpyAsync(b.d_reduce, red.data(), sizeof(irtps::ReduceObj) * red.size(), cudaMemcpyHostToDevice, b.stream),
         "partial-sum descriptors");
-  if ((rblk != b.reduce_blocks || (int)red.size() != b.n_reduce) && b.graph) {
+  if ((rblk != b.reduce_blocks || (int)red.size() != b.n_reduce || begin != b.n_items) && b.graph) {
     cudaGraphExecDestroy(b.graph);
     b.graph = nullptr;
   }
+  b.n_items = begin;
   b.reduce_blocks = rblk;
   b.n_reduce = (int)red.size();
   return IRTPS_OK;

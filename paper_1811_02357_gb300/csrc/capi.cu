@@ -181,6 +181,7 @@ int prepare_trace(Ctx &c, int n_pix, int spp) {
   if (need == 0) return IRTPS_OK;
   bool grown = false;
   const cudaError_t e = irtps::ensure_shared_scratch(c, need, grown);
+  if (e == cudaErrorMemoryAllocation && c.opt.sampling != 1) return IRTPS_OK;  // traced without the sample split
   if (e != cudaSuccess)
     return fail(c, e == cudaErrorMemoryAllocation ? IRTPS_ENOMEM : IRTPS_ECUDA,
                 std::string("trace partial sums: ") + cudaGetErrorString(e));

@@ -303,7 +303,8 @@ struct SharedSplit {
   int n_chunks, chunk;  // as in ObjTrace
 };
 SharedSplit shared_split(int n_pix, int spp);
-SharedSplit light_split(const Ctx &c, int spp);  // per-light sampling (one chunk unless the object is small)
+constexpr long long kSplitBytes = 256ll << 20;  // sample radiances of one call's split objects, at most
+SharedSplit light_split(const Ctx &c, int n_pix, int spp);  // per-light sampling (one chunk unless the object is small)
 cudaError_t ensure_shared_scratch(Ctx &c, size_t need, bool &grown);
 struct ReduceObj {
   float *part;     // as in ObjTrace

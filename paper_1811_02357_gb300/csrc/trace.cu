@@ -1,4 +1,4 @@
-// Reverted Monte-Carlo trace (Sec. IV, Eq. 5-7): min/max pyramid build, the
+// Reverted Monte-Carlo trace (Sec. IV, Eq. 5-7): pyramid build (maxima and bounding planes), the
 // trace kernel (per light or light-shared, single object or batched), the
 // stage-0 forward render, and geometry probes used by the parity tests.
 #include <algorithm>
@@ -403,7 +403,7 @@ __device__ __forceinline__ void env_lookup(const float *__restrict__ env, int EH
   }
 }
 
-// a / w correctly rounded for an integer w (1 to 2^14), inv = 1 / w rounded to nearest: with a correctly rounded
+// a / w correctly rounded for an integer w (1 to 2^15 + 1), inv = 1 / w rounded to nearest: with a correctly rounded
 // reciprocal, one correction of the quotient by its exact remainder rounds correctly (Markstein, "Computation of
 // elementary functions on the IBM RISC System/6000 processor", 1990, theorem on division); checked against the
 // division over every width in a CPU test.
@@ -425,7 +425,7 @@ __device__ __forceinline__ float div_width(float a, float w, float inv) {
 //
 // Execution: every lane is a small state machine (set up a segment -> march ->
 // resolve).  March steps of all lanes run in a loop that the warp leaves only
-// when at most half of its live lanes are still marching; the finished lanes
+// when at most a quarter of its live lanes are still marching; the finished lanes
 // then resolve and set up their next segments together.  Lanes therefore stay
 // busy although path lengths differ widely, while each lane's own sequence of
 // operations - and so every result bit - is that of a plain sequential trace.
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(kTraceThreads,
     return F3{__ldg(l), __ldg(l + 1), __ldg(l + 2)};
   };
   // march-loop iterations a segment may take (a lane waiting for its leaf step counts them too)
-  auto budget0 = [&]() -> int { return 32 * (ob->f.Wc + ob->f.Hc + 8) * (ob->f.levels + 1); };
+  auto budget0 = [&]() -> int { return 64 * (ob->f.Wc + ob->f.Hc + 8) * (ob->f.levels + 1); };
   const uint32_t iter_base = a.iter_dev ? *a.iter_dev : a.iter;
 
   int phase = PH_SETUP;
@@ -1037,12 +1037,8 @@ SharedSplit shared_split(int n_pix, int spp) {
 #ifndef IRTPS_SPLIT_MIN_CHUNK
 #define IRTPS_SPLIT_MIN_CHUNK 2
 #endif
-#ifndef IRTPS_SPLIT_MB
-#define IRTPS_SPLIT_MB 256
-#endif
-constexpr long long kSplitBytes = (long long)IRTPS_SPLIT_MB << 20;
-SharedSplit light_split(const Ctx &c, int spp) {
-  const long long items = (long long)c.H * c.W * c.K;
+SharedSplit light_split(const Ctx &c, int n_pix, int spp) {
+  const long long items = (long long)n_pix * c.K;
   long long n = (1ll << IRTPS_SPLIT_ITEMS_LOG2) / items;
   const long long most = spp / IRTPS_SPLIT_MIN_CHUNK;
   n = std::max(1ll, std::min(n, most));
@@ -1055,7 +1051,7 @@ SharedSplit light_split(const Ctx &c, int spp) {
 
 size_t trace_scratch_floats(const Ctx &c, int n_pix, int spp) {
   if (c.opt.sampling == 1) return (size_t)shared_split(n_pix, spp).n_chunks * (c.K + 1) * c.C * n_pix;
-  return light_split(c, spp).n_chunks > 1 ? (size_t)spp * c.K * c.C * n_pix : 0;
+  return light_split(c, n_pix, spp).n_chunks > 1 ? (size_t)spp * c.K * c.C * n_pix : 0;
 }
 
 cudaError_t launch_trace(Ctx &c, const int32_t *pixels, int n_pix, int spp, int bounces, uint64_t seed,
@@ -1091,11 +1087,11 @@ cudaError_t launch_trace(Ctx &c, const int32_t *pixels, int n_pix, int spp, int 
     if (cudaMemsetAsync(a.one.part, 0, sizeof(float) * lights, c.stream) != cudaSuccess) return cudaGetLastError();
     n = (long long)n_pix * a.one.n_chunks;
   } else {
-    const SharedSplit sp = light_split(c, spp);
+    SharedSplit sp = light_split(c, n_pix, spp);
+    if ((size_t)spp * c.K * c.C * n_pix > c.shared_cap) sp = {1, spp};  // no room for the radiances: unsplit, same bits
     a.one.n_chunks = sp.n_chunks;
     a.one.chunk = sp.chunk;
     if (sp.n_chunks > 1) {
-      if ((size_t)spp * c.K * c.C * n_pix > c.shared_cap) return cudaErrorInvalidValue;  // not prepared
       a.one.part = c.shared_part;
       if (a.one.hole && cudaMemsetAsync(a.one.hole, 1, (size_t)c.K * n_pix, c.stream) != cudaSuccess)
         return cudaGetLastError();
