@@ -24,8 +24,8 @@
 namespace irtps {
 
 enum Slot { S_BB = 0, S_PAP = 1, S_RZ0 = 2, S_RZ1 = 3, S_RR = 4, S_SUMX = 5, S_DMAX = 6, S_DSQ = 7, S_HMAX = 8,
-            S_HMIN = 9, S_RZREF = 10 };
-static_assert(S_RZREF < kPartSlots, "partial slots");
+            S_HMIN = 9, S_RS = 10 };
+static_assert(S_RS < kPartSlots, "partial slots");
 
 #ifndef IRTPS_CG_THREADS
 #define IRTPS_CG_THREADS 256
@@ -82,6 +82,20 @@ __device__ __forceinline__ double total(const double *part, int n, double *sh) {
   }
   __syncthreads();
   return sh[32];
+}
+
+// Two such sums at once (a block of at least two warps).
+__device__ __forceinline__ double2 total2(const double *a, const double *b, int n, double *sh) {
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    const double *part = threadIdx.x < 32 ? a : b;
+    double v = 0.0;
+    for (int i = threadIdx.x & 31; i < n; i += 32) v += part[i];
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x < 32 ? 32 : 31] = v;
+  }
+  __syncthreads();
+  return make_double2(sh[32], sh[31]);
 }
 
 template <typename T>
@@ -195,10 +209,7 @@ __device__ __forceinline__ void residual_body(const CG &g, int rz_slot, Team t) 
     rr += res * res;
   }
   rz = block_reduce<false>(rz, sh);
-  if (threadIdx.x == 0) {
-    g.part[rz_slot * g.stride + t.bid] = rz;
-    g.part[S_RZREF * g.stride + t.bid] = rz;
-  }
+  if (threadIdx.x == 0) g.part[rz_slot * g.stride + t.bid] = rz;
   rr = block_reduce<false>(rr, sh);
   if (threadIdx.x == 0) g.part[S_RR * g.stride + t.bid] = rr;
 }
@@ -469,11 +480,27 @@ __device__ void mg_vcycle(const MG &m, const float *r, CGCtl *ctl, Team t) {
 
 // z = A_1^+ r by the FP32 cosine transforms (A_1 the unit-weight Laplacian), a preconditioner of the weighted
 // solves: the Huber weights lie in (0, 1] and differ from 1 at a tenth of the edges, so PCG takes 16 to 21
-// iterations to 1e-9 whatever the grid, four barriers each, where the V-cycle takes some thirty barriers and
-// several times the iterations.  Called by all blocks with r complete; on return all of z is visible to all blocks.
-__device__ void spectral_solve(const SpecObj &o, const float *r, float *z, CGCtl *ctl, Team t) {
+// iterations to 1e-9 whatever the grid, where the V-cycle takes some thirty barriers and several times the
+// iterations.  With `update` the step comes first, e += af p, r -= af Ap: a block transforms the rows that it
+// updates, which saves a pass and a barrier.  Returns the thread's sums of r.z and (with `update`) of (rscale r)^2.
+// Two barriers; the caller's next one publishes z.  One copy in the code (the FFT stages are long).
+// With the step inside, no solve for a residual about to be refreshed, and the refresh by the FP32 residual, classic PS
+// and three reweightings at 375 x 421 went from 5.13 to 4.50 ms.
+__device__ __noinline__ float2 spectral_solve(const SpecObj &o, const CG &g, float *e, bool update, float af,
+                                              const float *p, float rscale, CGCtl *ctl, Team t) {
+  float rz = 0.0f, rs = 0.0f;
   for (int i = t.bid; i < o.row_blocks; i += t.nblk) {
-    spec::rows_forward<spec::SRC_ARRAY>(o, i, r);
+    spec::rows_forward<spec::SRC_CALL>(o, i, [&](size_t q) {
+      float r = g.r[q];
+      if (update) {
+        e[q] = fmaf(af, p[q], e[q]);
+        r = fmaf(-af, g.ap[q], r);
+        g.r[q] = r;
+        const float u = r * rscale;
+        rs = fmaf(u, u, rs);
+      }
+      return r;
+    });
     __syncthreads();
   }
   grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
@@ -483,10 +510,13 @@ __device__ void spectral_solve(const SpecObj &o, const float *r, float *z, CGCtl
   }
   grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
   for (int i = t.bid; i < o.row_blocks; i += t.nblk) {
-    spec::rows_back<spec::DST_ARRAY>(o, i, z);
+    spec::rows_back<spec::DST_CALL>(o, i, [&](size_t q, float z) {
+      g.z[q] = z;
+      rz = fmaf(g.r[q], z, rz);
+    });
     __syncthreads();
   }
-  grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+  return make_float2(rz, rs);
 }
 
 // The whole PCG loop in one cooperative launch (PRE 0: Jacobi, M = diag(degree);
@@ -501,9 +531,10 @@ __device__ void spectral_solve(const SpecObj &o, const float *r, float *z, CGCtl
 // value at the last refresh (the FP32 recursion has converged and further steps
 // would follow rounding noise: the direction is then frozen to 0), x64 += e,
 // e = 0, and the residual is recomputed in FP64 (r = b - A x64) and tested
-// against tol (iterative refinement).  Dot products are FP32 within a block and
-// FP64 across blocks; every block sums the same partials in the same order and
-// so takes the same decisions.
+// against tol (iterative refinement); only a solve that goes on applies the preconditioner again.  PRE 2 also
+// refreshes when the FP32 residual falls below tol / 2, since its iterations are few and dear.
+// Dot products are FP32 within a block and FP64 across blocks; every block sums the same partials in the same
+// order and so takes the same decisions.
 template <int PRE, bool WEIGHTED>
 __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc, double tol, int max_iter, int check,
                                              const MG &mg, const SpecObj *so, Team t) {
@@ -519,40 +550,94 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
   float *e = g.ap + g.P;  // correction accumulator (second half of the Ap buffer)
   float *z = PRE == 1 ? mg.x1 : g.z;  // preconditioned residual (level 0 of the hierarchy for PRE 1)
   for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) e[q.p] = 0.0f;
-  // z = M^-1 r and the partial sums of r.z into `slot` (and the refresh reference)
-  auto precondition = [&](int slot, bool refresh) {
-    if (PRE != 0) grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);  // r complete
-    if (PRE == 1) mg_vcycle(mg, g.r, ctl, t);
-    if (PRE == 2) spectral_solve(*so, g.r, g.z, ctl, t);
-    float rz = 0.0f;
-    for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
-      const float rf = g.r[q.p];
-      float zf;
-      if (PRE != 0) {
-        zf = z[q.p];
-      } else {
-        zf = WEIGHTED ? rf / weighted_degree(g.wh, g.wv, q.p, q.i, q.j, g.H, g.W)
-                      : rf * inv_degree(q.i, q.j, g.H, g.W);
-        z[q.p] = zf;
+  // z = M^-1 r and the partial sums of r.z into `slot`; r is complete at the call.
+  // PRE 2 with `update`: after e += af p, r -= af Ap, and with the partial sums of (r / (tol |b|))^2.
+  const float rscale = (float)(1.0 / (tol * bnorm));
+  auto precondition = [&](int slot, bool update, float af, const float *p) {
+    float rz = 0.0f, rs = 0.0f;
+    if (PRE == 2) {
+      const float2 v = spectral_solve(*so, g, e, update, af, p, rscale, ctl, t);
+      rz = v.x;
+      rs = v.y;
+    } else {
+      if (PRE == 1) mg_vcycle(mg, g.r, ctl, t);
+      for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
+        const float rf = g.r[q.p];
+        float zf;
+        if (PRE != 0) {
+          zf = z[q.p];
+        } else {
+          zf = WEIGHTED ? rf / weighted_degree(g.wh, g.wv, q.p, q.i, q.j, g.H, g.W)
+                        : rf * inv_degree(q.i, q.j, g.H, g.W);
+          z[q.p] = zf;
+        }
+        rz = fmaf(rf, zf, rz);
       }
-      rz = fmaf(rf, zf, rz);
     }
     rz = block_sum_f(rz, shf);
-    if (threadIdx.x == 0) {
-      g.part[slot * g.stride + t.bid] = (double)rz;
-      if (refresh) g.part[S_RZREF * g.stride + t.bid] = (double)rz;
+    if (threadIdx.x == 0) g.part[slot * g.stride + t.bid] = (double)rz;
+    if (PRE == 2 && update) {
+      rs = block_sum_f(rs, shf);
+      if (threadIdx.x == 0) g.part[S_RS * g.stride + t.bid] = (double)rs;
     }
   };
+  // Refresh from FP64: x64 += e, e = 0, r = b - A x64, its norm against tol, and z, r.z of iteration `it` unless the
+  // solve ends here (returned).  `af`: the step along p that e still lacks.
+  auto refresh = [&](float af, const float *p) -> bool {
+    for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
+      g.x[q.p] += (double)fmaf(af, p[q.p], e[q.p]);
+      e[q.p] = 0.0f;
+    }
+    grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+    if (*(volatile int *)&ctl->err) return true;
+    double rr = 0.0;
+    for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
+      const double ax = WEIGHTED ? lap_weighted<double>(g.x, g.wh, g.wv, q.i, q.j, g.H, g.W)
+                                 : lap_at<double>(g.x, q.i, q.j, g.H, g.W);
+      const double res = g.b[q.p] - ax;
+      g.r[q.p] = (float)res;
+      rr += res * res;
+    }
+    rr = block_reduce<false>(rr, sh);
+    if (threadIdx.x == 0) g.part[S_RR * g.stride + t.bid] = rr;
+    if (PRE == 0) precondition(S_RZ0 + (it & 1), false, 0.0f, nullptr);  // cheaper than a second barrier
+    grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+    if (*(volatile int *)&ctl->err) return true;
+    rel = sqrt(total(g.part + S_RR * g.stride, g.nblk, sh)) / bnorm;
+    if (!isfinite(rel) || !(rel > tol)) return true;
+    if (rel < 0.95 * best) {
+      best = rel;
+      stall = it;
+    } else if (it - stall >= 1000) {
+      return true;  // no 5% gain in 1000 iterations: the FP64 residual is at its rounding floor
+    }
+    if (PRE == 0) return false;
+    precondition(S_RZ0 + (it & 1), false, 0.0f, nullptr);
+    grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+    return *(volatile int *)&ctl->err != 0;
+  };
   if (PRE != 0 && rel > tol) {  // the residual kernel left r; z and r.z come from the preconditioner
-    precondition(S_RZ0, true);
+    precondition(S_RZ0, false, 0.0f, nullptr);
     grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
   }
+  double num = 0.0, ref = 0.0;  // r.z of the last iteration and of the last refresh
+  int fresh = 0;                // the iteration of the last refresh
   while (rel > tol && it < max_iter && !*(volatile int *)&ctl->err) {
-    ++it;
     // ---- A ----
-    const double num = total(g.part + (S_RZ0 + ((it - 1) & 1)) * g.stride, g.nblk, sh);
-    const double ref = total(g.part + S_RZREF * g.stride, g.nblk, sh);
-    const double den = it > 1 ? total(g.part + (S_RZ0 + (it & 1)) * g.stride, g.nblk, sh) : 0.0;
+    const double den = num;
+    if (PRE == 2 && it >= fresh + 3) {  // refresh once the FP32 residual says that the solve is done
+      const double2 s = total2(g.part + (S_RZ0 + (it & 1)) * g.stride, g.part + S_RS * g.stride, g.nblk, sh);
+      num = s.x;
+      if (s.y <= 0.25) {
+        fresh = it;
+        if (refresh(0.0f, e)) break;
+        num = total(g.part + (S_RZ0 + (it & 1)) * g.stride, g.nblk, sh);
+      }
+    } else {
+      num = total(g.part + (S_RZ0 + (it & 1)) * g.stride, g.nblk, sh);
+    }
+    if (it == fresh) ref = num;
+    ++it;
     if (threadIdx.x == 0) {
       const bool frozen = !(num > 1e-10 * ref);
       s_frozen = frozen;
@@ -595,44 +680,22 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
     if (threadIdx.x == 0) s_ab[0] = (dpap > 0.0 && isfinite(dpap)) ? (float)(num / dpap) : 0.0f;
     __syncthreads();
     const float af = s_ab[0];
-    for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
-      const int p = q.p;
-      e[p] = fmaf(af, pnew[p], e[p]);
-      g.r[p] = fmaf(-af, g.ap[p], g.r[p]);
+    if (it % check == 0 || frozen) {  // r comes from FP64
+      fresh = it;
+      if (refresh(af, pnew)) break;
+      continue;
     }
-    precondition(S_RZ0 + (it & 1), false);
+    if (PRE != 2) {
+      for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
+        const int p = q.p;
+        e[p] = fmaf(af, pnew[p], e[p]);
+        g.r[p] = fmaf(-af, g.ap[p], g.r[p]);
+      }
+      if (PRE != 0) grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);  // r complete
+    }
+    precondition(S_RZ0 + (it & 1), true, af, pnew);
     grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
     if (*(volatile int *)&ctl->err) break;
-    // ---- refresh from FP64 ----
-    if (it % check == 0 || frozen) {
-      for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
-        g.x[q.p] += (double)e[q.p];
-        e[q.p] = 0.0f;
-      }
-      grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
-      if (*(volatile int *)&ctl->err) break;
-      double rr = 0.0;
-      for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
-        const double ax = WEIGHTED ? lap_weighted<double>(g.x, g.wh, g.wv, q.i, q.j, g.H, g.W)
-                                   : lap_at<double>(g.x, q.i, q.j, g.H, g.W);
-        const double res = g.b[q.p] - ax;
-        g.r[q.p] = (float)res;
-        rr += res * res;
-      }
-      rr = block_reduce<false>(rr, sh);
-      if (threadIdx.x == 0) g.part[S_RR * g.stride + t.bid] = rr;
-      precondition(S_RZ0 + (it & 1), true);
-      grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
-      if (*(volatile int *)&ctl->err) break;
-      rel = sqrt(total(g.part + S_RR * g.stride, g.nblk, sh)) / bnorm;
-      if (!isfinite(rel)) break;
-      if (rel < 0.95 * best) {
-        best = rel;
-        stall = it;
-      } else if (it - stall >= 1000) {
-        break;  // no 5% gain in 1000 iterations: the FP64 residual is at its rounding floor
-      }
-    }
   }
   // fold in a correction collected since the last refresh (none when the loop ended on a refresh)
   for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) g.x[q.p] += (double)e[q.p];

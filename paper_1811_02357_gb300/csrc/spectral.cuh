@@ -277,20 +277,23 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
 
 extern __shared__ __align__(16) float2 spec_smem[];
 
-// Rows forward: two rows per block, of b (from the normals, kept; |b|^2 partials), of the residual, or of a FP32
-// array v.
-enum : int { SRC_RHS = 0, SRC_RESIDUAL = 1, SRC_ARRAY = 2 };
-template <int SRC>
-__device__ __forceinline__ void rows_forward(const SpecObj &o, int blk, const float *v0 = nullptr) {
+// Rows forward: two rows per block, of b (from the normals, kept; |b|^2 partials), of the residual, or of the values
+// load(p) of the pixels.
+struct NoCall {
+  __device__ float operator()(size_t, float = 0.0f) const { return 0.0f; }
+};
+enum : int { SRC_RHS = 0, SRC_RESIDUAL = 1, SRC_CALL = 2 };
+template <int SRC, class F = NoCall>
+__device__ __forceinline__ void rows_forward(const SpecObj &o, int blk, F load = F()) {
   const FftPlan &P = o.row;
   const int n = o.W, i0 = 2 * blk;
   const bool two = i0 + 1 < o.H;
   float2 *a = spec_smem, *b = a + line_stride(P.m);
   double bb = 0.0;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    if (SRC == SRC_ARRAY) {
-      const float *r = v0 + (size_t)i0 * n + j;
-      a[at(place(j, n))] = make_float2(r[0], two ? r[n] : 0.0f);
+    if (SRC == SRC_CALL) {
+      const size_t p = (size_t)i0 * n + j;
+      a[at(place(j, n))] = make_float2(load(p), two ? load(p + n) : 0.0f);
       continue;
     }
     double u, v = 0.0;
@@ -374,10 +377,10 @@ __device__ __forceinline__ void columns(const SpecObj &o, int blk, int L) {
 }
 
 // Rows back: two rows per block, into the FP64 iterate (set, or added to; the last one's partial sums give the
-// mean), or into a FP32 array v.
-enum : int { DST_SET = 0, DST_ADD = 1, DST_ADD_LAST = 2, DST_ARRAY = 3 };
-template <int DST>
-__device__ __forceinline__ void rows_back(const SpecObj &o, int blk, float *v0 = nullptr) {
+// mean), or handed to store(p, value).
+enum : int { DST_SET = 0, DST_ADD = 1, DST_ADD_LAST = 2, DST_CALL = 3 };
+template <int DST, class F = NoCall>
+__device__ __forceinline__ void rows_back(const SpecObj &o, int blk, F store = F()) {
   constexpr bool FIRST = DST == DST_SET, LAST = DST == DST_ADD_LAST;
   const FftPlan &P = o.row;
   const int n = o.W, i0 = 2 * blk;
@@ -395,10 +398,10 @@ __device__ __forceinline__ void rows_back(const SpecObj &o, int blk, float *v0 =
   double sum = 0.0;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     const float2 v = z[at(place(j, n))];
-    if (DST == DST_ARRAY) {
-      float *r = v0 + (size_t)i0 * n + j;
-      r[0] = v.y;
-      if (two) r[n] = v.x;
+    if (DST == DST_CALL) {
+      const size_t p = (size_t)i0 * n + j;
+      store(p, v.y);
+      if (two) store(p + n, v.x);
       continue;
     }
     const double ua = FIRST ? (double)v.y : xa[j] + (double)v.y;

@@ -96,3 +96,23 @@ def test_weighted_batch_mixes_preconditioners(lib):
         c.close()
     for s, g in zip(single, got):
         assert np.abs(g - s).max() <= 1e-4 * np.ptp(s)
+
+
+@pytest.mark.parametrize("precond", [0, 1, 2])
+@pytest.mark.parametrize("every,tol", [(1, 1e-9), (2, 1e-6), (7, 1e-9), (1000, 1e-9), (1000, 1e-3)])
+def test_refresh_rules_of_weighted_solves(lib, oracle_mod, precond, every, tol):
+    """Whenever the residual is refreshed (every so many iterations, or when the FP32 recursion says so), a solve ends
+    on an FP64 residual within its tolerance; at 1e-9 the surface is the oracle's."""
+    H, W = 61, 53
+    n = _normals(H, W)
+    n[20:24, 10:30] = np.array([0.6, 0.0, 0.8], np.float32)
+    opt = lib.irtps_default_options()
+    opt.irls_iters, opt.precond, opt.cg_check_every, opt.cg_tol = 2, precond, every, tol
+    with lib.Context(H, W, scenes.ring_lights(3, 45.0), np.zeros((1, 2, 2), np.float32), opt) as ctx:
+        ctx.set_state(depth=np.zeros((H, W), np.float32), normals=n)
+        ctx.integrate()
+        d, st = ctx.depth(), ctx.stats()
+    assert 0 < st["cg_rel_residual"] <= tol
+    if tol == 1e-9:
+        want = oracle_mod.irls_solve(n.astype(np.float64), 1.0 / W, 0.05, 2)
+        assert np.abs(d - want).max() <= 1e-4 * np.ptp(want)
