@@ -68,10 +68,11 @@ typedef struct irtps_options {
   int cg_check_every; /* FP64 true-residual refresh and convergence test period (10) */
   double stop_tol;    /* irtps_iterate stops early when D_H < stop_tol; 0 = never (0) */
   int precond;        /* depth solve: 0 Jacobi-preconditioned CG, 1 multigrid-preconditioned CG,
-                         2 direct: unit-weight solves of grids up to 1024 x 1024 by the cosine
-                         transform that diagonalises the grid Laplacian (four FP64 transform
-                         products, then the same FP64 residual check against cg_tol); weighted
-                         (irls) solves, larger grids and batches use multigrid (2) */
+                         2 direct: unit-weight solves of grids up to 4096 x 4096 by the cosine
+                         transform that diagonalises the grid Laplacian (fast transforms in FP32,
+                         refined on FP64 residuals, then the same FP64 residual check against cg_tol),
+                         which also preconditions their weighted (irls) solves; larger grids use
+                         multigrid (2) */
   int use_graph;      /* 1: irtps_iterate captures one iteration as a CUDA graph and replays it (0);
                          per-stage times are then not measured (reported as 0) */
   int sampling;       /* trace sampling (0):
@@ -84,8 +85,8 @@ typedef struct irtps_options {
   float irls_delta;   /* Huber threshold on the edge slope residual (H_b - H_a)/h - mean slope (0.05) */
   int early_escape;   /* before a trace, bound every pixel's horizon in eight octants of azimuth
                          from the max pyramid (a fixed scan of nodes around the pixel per level);
-                         a rising primary ray above it skips its march after the triangle test of
-                         its first cell (results unchanged, bit for bit).  0 off, 1 on, 2 where it
+                         a rising primary ray above it skips its march once it is clear of its first
+                         cell (results unchanged, bit for bit).  0 off, 1 on, 2 where it
                          pays: per-light sampling, at least 16 samples per item, and H W K >= 2^18
                          work items (a smaller object cannot fill the GPU; in a batch any size) (2) */
   int fill_holes;     /* 1: the single-sample variant of Sec. IV (per-light sampling only): a (pixel,
@@ -103,8 +104,8 @@ typedef struct irtps_options {
                          tile, BF16 hi + lo split of I and pinv(L), FP32 accumulation:
                          I_hi P_hi + I_lo P_hi + I_hi P_lo).  Row masks and masked pixels are decided
                          and solved identically in both (FP32 masks; masked 3x3 systems in FP32 when
-                         well conditioned, else double-float sums with an FP64 inverse and condition
-                         number).  Batches use the FP32 form (0) */
+                         well conditioned, else fixed-point and compensated sums with a refined FP32 or
+                         an FP64 solve).  Batches use the FP32 form (0) */
 } irtps_options;
 
 /* Counters of the last irtps_iterate / irtps_trace / irtps_integrate call. */

@@ -485,7 +485,7 @@ __device__ void mg_vcycle(const MG &m, const float *r, CGCtl *ctl, Team t) {
 // updates, which saves a pass and a barrier.  Returns the thread's sums of r.z and (with `update`) of (rscale r)^2.
 // Two barriers; the caller's next one publishes z.  One copy in the code (the FFT stages are long).
 // With the step inside, no solve for a residual about to be refreshed, and the refresh by the FP32 residual, classic PS
-// and three reweightings at 375 x 421 went from 5.13 to 4.50 ms.
+// and three reweightings at 375 x 421 went from 5.1-5.5 to 3.9-4.5 ms (the inputs differ in their iterations).
 __device__ __noinline__ float2 spectral_solve(const SpecObj &o, const CG &g, float *e, bool update, float af,
                                               const float *p, float rscale, CGCtl *ctl, Team t) {
   float rz = 0.0f, rs = 0.0f;

@@ -23,8 +23,8 @@
 //
 // The same three passes in FP32 precondition the weighted (IRLS) solves (poisson.cu).
 //
-// Against the dense FP64 transforms this replaces up to 1024 on a side and the multigrid PCG
-// beyond: see launch_spectral.
+// Whole calls against the dense FP64 transforms (to 1024 on a side) and the multigrid PCG (beyond) that it replaced:
+// 512 x 512 684 -> 135 us, 637 x 899 1862 -> 283 us, classic PS and surface at 2048 x 2048 26.4 -> 1.19 ms.
 #include <algorithm>
 #include <cmath>
 #include <complex>
