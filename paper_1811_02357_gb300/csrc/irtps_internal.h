@@ -271,6 +271,10 @@ constexpr int kSpectralMaxSide = 4096;
 bool spectral_fits(int H, int W);
 cudaError_t spectral_setup(Ctx &c);   // plans and work array
 SpecObj spec_object(const Ctx &c, CGAcc *acc);
+// Lets a kernel be launched with all the dynamic shared memory that a block may have on this device.  The limit
+// belongs to the function and not to a context, so it is set to this one value wherever it is set: a size of the
+// caller's own would refuse the launches of other threads' contexts that take more.
+cudaError_t allow_max_smem(const void *kernel);
 size_t spec_line_smem(const Ctx &c);  // shared memory of one line pair, rows or columns
 cudaError_t launch_spectral(Ctx &c);  // the whole solve: normals -> b, x, depth, residual check
 // whether a context's unit-weight solves are direct (option precond = 2 on a grid the transform covers)
@@ -330,6 +334,7 @@ cudaError_t launch_ps_batch(cudaStream_t s, int C, int dtype, const void *d_args
 cudaError_t solve_depth_async(Ctx &c);  // enqueue one depth solve (results accumulate in dstats->cg)
 cudaError_t depth_change_async(Ctx &c);  // enqueue D_H of depth against depth_prev into dstats
 int solve_depth(Ctx &c);                 // one solve, waited for (IRTPS_OK or an error code, message in c.err)
+cudaError_t cg_allow_smem();  // shared-memory limit of the weighted spectral solve's kernel (before its first use)
 int cg_grid_limit();  // co-resident blocks available to the cooperative solve
 // batched solves: one job per object, teams of blocks in one launch per step
 size_t cg_job_bytes();

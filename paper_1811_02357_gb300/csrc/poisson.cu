@@ -992,10 +992,8 @@ static cudaError_t solve_once(Ctx &c) {
   const bool spectral = WEIGHTED && direct_solve(c);
   const size_t smem = spectral ? spec_line_smem(c) : 0;
   if (spectral) {  // the cooperative grid that fits with the lines in shared memory
-    cudaError_t e =
-        cudaFuncSetAttribute(k_cg_loop_spectral, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cg_loop_spectral, kThreads, smem);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cg_loop_spectral, kThreads, smem);
     if (e != cudaSuccess) return e;
     if (per < 1) return cudaErrorInvalidConfiguration;
     g.nblk = std::min(g.nblk, per * (c.sms > 0 ? c.sms : 1));
@@ -1197,6 +1195,8 @@ __global__ void __launch_bounds__(kThreads) k_zero_depth_b(const CGJob *jobs, in
   });
 }
 
+cudaError_t cg_allow_smem() { return allow_max_smem((const void *)k_cg_loop_spectral); }
+
 size_t cg_job_bytes() { return sizeof(CGJob); }
 
 // Co-resident blocks of the batched solve loop (at most IRTPS_CG_BATCH_BLOCKS_PER_SM per SM).
@@ -1206,9 +1206,7 @@ int cg_batch_grid_limit(size_t smem) {
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
   int per_w = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cg_loop_b<false>, kThreads, 0) != cudaSuccess) return 0;
-  if (smem > 0 && cudaFuncSetAttribute(k_cg_loop_b<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-                      cudaSuccess)
-    return 0;
+  if (smem > 0 && allow_max_smem((const void *)k_cg_loop_b<true>) != cudaSuccess) return 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_w, k_cg_loop_b<true>, kThreads, smem) != cudaSuccess) return 0;
   per = per < per_w ? per : per_w;
   per = per < IRTPS_CG_BATCH_BLOCKS_PER_SM ? per : IRTPS_CG_BATCH_BLOCKS_PER_SM;
@@ -1253,11 +1251,6 @@ static cudaError_t solve_batch_once(cudaStream_t s, const CGJob *jobs, int n, in
   k_cg_start_b<WEIGHTED><<<n, 32, 0, s>>>(jobs);
   LAUNCH_CHECK();
   void *args[] = {(void *)&jobs, (void *)&n};
-  if (WEIGHTED && smem > 0) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_cg_loop_b<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_cg_loop_b<WEIGHTED>, dim3(blocks), dim3(kThreads), args,
                                               WEIGHTED ? smem : 0, s);
   if (e != cudaSuccess) return e;

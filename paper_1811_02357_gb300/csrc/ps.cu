@@ -954,7 +954,7 @@ cudaError_t launch_ps_batch(cudaStream_t s, int C, int dtype, const void *d_args
 template <int C, typename TI>
 static cudaError_t launch_ps_tc_t(Ctx &c, const PSArgs &a) {
   const size_t smem = tc_smem_bytes(c.K, C);
-  cudaError_t e = cudaFuncSetAttribute(k_ps_tc<C, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_max_smem((const void *)k_ps_tc<C, TI>);
   if (e != cudaSuccess) return e;
   // CTAs per SM from the shared-memory fit (the operands are most of a CTA's footprint; the
   // occupancy query answered one for this kernel).  The CTAs never wait on one another, and 4 of

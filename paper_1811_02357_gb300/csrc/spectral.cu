@@ -174,13 +174,17 @@ size_t col_smem(const SpecObj &o) { return sizeof(float2) * 2 * o.col_lines * li
 // tolerances get four, down to the floor of FP64.
 int refinements(const SpecObj &o) { return o.tol < 1e-10 ? 4 : (std::max(o.H, o.W) <= 128 ? 1 : 2); }
 
-template <typename F>
-cudaError_t allow_smem(F *k, size_t bytes) {
-  return bytes > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
-                           : cudaSuccess;
-}
-
 }  // namespace
+
+cudaError_t allow_max_smem(const void *kernel) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+}
 
 bool spectral_fits(int H, int W) { return H <= kSpectralMaxSide && W <= kSpectralMaxSide; }
 
@@ -205,7 +209,13 @@ cudaError_t spectral_setup(Ctx &c) {
   o.col_blocks = (W + 2 * o.col_lines - 1) / (2 * o.col_lines);
   const size_t pb = sizeof(float2) * pool.size(), lb = (sizeof(float) * lam.size() + 15) / 16 * 16;
   const size_t qb = sizeof(double) * (2 * o.row_blocks + o.check_blocks);
-  cudaError_t e = cudaMalloc(&c.sp_pool, pb + lb + qb);
+  cudaError_t e = cudaSuccess;
+  for (const void *k : {(const void *)k_spec<SP_ROWS_FIRST>, (const void *)k_spec<SP_ROWS>, (const void *)k_spec<SP_COLS>,
+                        (const void *)k_spec<SP_BACK_FIRST>, (const void *)k_spec<SP_BACK>,
+                        (const void *)k_spec<SP_BACK_LAST>})
+    if ((e = allow_max_smem(k)) != cudaSuccess) return e;
+  if (c.opt.irls_iters > 0 && (e = cg_allow_smem()) != cudaSuccess) return e;
+  e = cudaMalloc(&c.sp_pool, pb + lb + qb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c.sp_t, sizeof(float) * (size_t)H * W);
   if (e != cudaSuccess) return e;
   char *d = (char *)c.sp_pool;
@@ -252,12 +262,6 @@ size_t spec_line_smem(const Ctx &c) {
 cudaError_t launch_spectral(Ctx &c) {
   const SpecObj o = spec_object(c, &c.dstats->cg);
   const size_t rs = row_smem(o), cs = col_smem(o);
-  cudaError_t e;
-  if ((e = allow_smem(k_spec<SP_ROWS_FIRST>, rs)) != cudaSuccess || (e = allow_smem(k_spec<SP_ROWS>, rs)) != cudaSuccess ||
-      (e = allow_smem(k_spec<SP_BACK_FIRST>, rs)) != cudaSuccess || (e = allow_smem(k_spec<SP_BACK>, rs)) != cudaSuccess ||
-      (e = allow_smem(k_spec<SP_BACK_LAST>, rs)) != cudaSuccess ||
-      (e = allow_smem(k_spec<SP_COLS>, cs)) != cudaSuccess)
-    return e;
   cudaStream_t s = c.stream;
   k_spec<SP_ROWS_FIRST><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
   k_spec<SP_COLS><<<o.col_blocks, kColThreads, cs, s>>>(o);
@@ -297,7 +301,12 @@ cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, S
     ++sb.n;
   }
   if (sb.n == 0) return cudaSuccess;
-  cudaError_t e = cudaMalloc(&sb.table, sizeof(SpecObj) * sb.n);
+  cudaError_t e = cudaSuccess;
+  for (const void *k : {(const void *)k_spec_b<SP_ROWS_FIRST>, (const void *)k_spec_b<SP_ROWS>,
+                        (const void *)k_spec_b<SP_COLS>, (const void *)k_spec_b<SP_BACK_FIRST>,
+                        (const void *)k_spec_b<SP_BACK>, (const void *)k_spec_b<SP_BACK_LAST>})
+    if ((e = allow_max_smem(k)) != cudaSuccess) return e;
+  e = cudaMalloc(&sb.table, sizeof(SpecObj) * sb.n);
   if (e != cudaSuccess) return e;
   return cudaMemcpy(sb.table, t.data(), sizeof(SpecObj) * sb.n, cudaMemcpyHostToDevice);
 }
@@ -309,13 +318,6 @@ cudaError_t launch_spectral_batch(cudaStream_t s, const SpectralBatch &sb) {
   const SpecObj *t = (const SpecObj *)sb.table;
   const int n = sb.n;
   const size_t rs = sb.row_smem, cs = sb.col_smem;
-  cudaError_t e;
-  if ((e = allow_smem(k_spec_b<SP_ROWS_FIRST>, rs)) != cudaSuccess ||
-      (e = allow_smem(k_spec_b<SP_ROWS>, rs)) != cudaSuccess ||
-      (e = allow_smem(k_spec_b<SP_BACK_FIRST>, rs)) != cudaSuccess ||
-      (e = allow_smem(k_spec_b<SP_BACK>, rs)) != cudaSuccess ||
-      (e = allow_smem(k_spec_b<SP_BACK_LAST>, rs)) != cudaSuccess || (e = allow_smem(k_spec_b<SP_COLS>, cs)) != cudaSuccess)
-    return e;
   k_spec_b<SP_ROWS_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
   k_spec_b<SP_COLS><<<sb.blocks[1], kColThreads, cs, s>>>(t, n);
   k_spec_b<SP_BACK_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);

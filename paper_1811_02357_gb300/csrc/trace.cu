@@ -1307,10 +1307,7 @@ __global__ void k_render(const ObjTrace a, const float *__restrict__ lbar, float
 // else the per-light one.
 template <typename F>
 static int grid_of(F kernel, size_t smem, int sms) {
-  int per = 0;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 0;
+  int per = 0;  // (the tables of 64 objects take 10 KB: no shared-memory limit to raise)
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kTraceThreads, smem) != cudaSuccess) return 0;
   return per * sms;
 }
