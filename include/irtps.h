@@ -70,7 +70,8 @@ typedef struct irtps_options {
   int precond;        /* depth solve: 0 Jacobi-preconditioned CG, 1 multigrid-preconditioned CG,
                          2 direct: unit-weight solves of grids up to 4096 x 4096 by the cosine
                          transform that diagonalises the grid Laplacian (fast transforms in FP32,
-                         refined on FP64 residuals, then the same FP64 residual check against cg_tol),
+                         refined until the FP64 residual is within cg_tol or falls no further; one
+                         iteration in the statistics),
                          which also preconditions their weighted (irls) solves; larger grids use
                          multigrid (2) */
   int use_graph;      /* 1: irtps_iterate captures one iteration as a CUDA graph and replays it (0);

@@ -508,9 +508,10 @@ int irtps_batch_create(irtps_batch **out, irtps_ctx *const *objs, int n_obj, int
   {
     std::vector<Ctx *> cs;
     for (int i = 0; i < n_obj; ++i) cs.push_back(&objs[i]->c);
-    if (irtps::spectral_batch_setup(cs, b.d_stats, b.spectral) != cudaSuccess) {
+    const cudaError_t e = irtps::spectral_batch_setup(cs, b.d_stats, b.spectral);
+    if (e != cudaSuccess) {
       cudaGetLastError();
-      return bail(IRTPS_ENOMEM);
+      return bail(e == cudaErrorMemoryAllocation ? IRTPS_ENOMEM : IRTPS_ECUDA);
     }
   }
   if (cudaMemcpy(b.d_pyr, pyr.data(), sizeof(irtps::PyrObj) * n_obj, cudaMemcpyHostToDevice) != cudaSuccess ||

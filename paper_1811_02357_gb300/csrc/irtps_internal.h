@@ -104,14 +104,14 @@ struct SpecObj {
   float *depth;
   double *b, *x;         // right-hand side, iterate (H x W)
   float *t;              // spectrum (H x W)
-  double *part;          // partial sums: row_blocks of |b|^2, row_blocks of x, check_blocks of |r|^2
+  double *part;          // partial sums: row_blocks of |b|^2, row_blocks of x, check_blocks of |r|^2 (last pass)
   CGCtl *ctl;
   CGAcc *acc;
   FftPlan row, col;      // lengths W and H
   const float *mu, *nu;  // eigenvalues of the columns' and rows' path Laplacians
   int row_blocks, col_blocks, check_blocks;
   int col_lines;         // complex lines (pairs of columns) per block of the column pass
-  int blk[3];            // first block in a batched launch: row, column, check passes
+  int blk[3];            // first block in a batched launch: row, column, last passes
 };
 
 struct Ctx {
@@ -282,9 +282,9 @@ inline bool direct_solve(const Ctx &c) { return c.opt.precond == 2 && c.sp_t != 
 // the direct solves of a batch's objects: descriptors in one device table
 struct SpectralBatch {
   int n = 0;              // objects with direct solves
-  int blocks[3] = {0};    // row, column, check passes
+  int blocks[3] = {0};    // row, column, last passes
   int refine = 0;         // refinement steps
-  size_t row_smem = 0, col_smem = 0;
+  size_t row_smem = 0, col_smem = 0, line_smem = 0;
   void *table = nullptr;  // owned
 };
 cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, SpectralBatch &sb);

@@ -12,12 +12,14 @@
 // complex FFT of n points over two lines at once (one in the real, one in the imaginary
 // part; even samples ascending, then odd ones descending), held in shared memory, so a
 // solve is three passes over the grid: rows forward, columns forward - divided by the
-// eigenvalues - and back, rows back.  One such solve has a relative residual of about
-// 1e-3 at 2048 x 2048 (the rounding of x in FP32 against the second differences in b);
-// the FP64 residual r = b - A x, solved for the same way and added to the FP64 iterate,
-// lowers it by 1e-4 or more a step (a rough r needs little of x's range), so three solves
-// end below 1e-10, where FP64 transforms end too, while GB300's FP64 pipe (2
-// multiply-adds per clock and SM) does only the 13 operations of the residual per pixel.
+// eigenvalues - and back, rows back.  One such solve leaves a relative residual that grows with
+// the square of the longer side and with the smoothness of the slopes (the rounding of x in FP32
+// against the second differences in b): 1e-3 with noise, 0.1 without for 2048 points.  The FP64
+// residual r = b - A x, solved for the same way and added to the FP64 iterate, lowers it step by
+// step (2048 x 2048, noise-free slopes of the lowest modes: 0.1, 3e-8, 4e-10, 9e-11; the last
+// is the rounding of the FP64 residual), while GB300's FP64 pipe (2 multiply-adds per clock and SM)
+// does only the 14 operations of the residual per pixel.  One or two steps are launched ahead; the last
+// pass measures the residual and takes more where it is still above the tolerance (finish).
 // The slopes in b are quotients of FP32 numbers: FP32 quotient plus FP32 remainder
 // quotient (48 bits) instead of FP64 divisions.
 //
@@ -34,6 +36,7 @@
 
 #include "irtps_internal.h"
 #include "spectral.cuh"
+#include "team.cuh"
 
 namespace irtps {
 
@@ -43,7 +46,7 @@ using namespace spec;
 
 constexpr int kMaxSmem = 227 * 1024;
 
-enum : int { SP_ROWS_FIRST = 0, SP_ROWS = 1, SP_COLS = 2, SP_BACK_FIRST = 3, SP_BACK = 4, SP_BACK_LAST = 5, SP_CHECK = 6 };
+enum : int { SP_ROWS_FIRST = 0, SP_ROWS = 1, SP_COLS = 2, SP_BACK_FIRST = 3, SP_BACK = 4, SP_BACK_LAST = 5 };
 template <int PASS>
 __device__ __forceinline__ void spec_pass(const SpecObj &o, int blk) {
   if (PASS == SP_ROWS_FIRST) rows_forward<SRC_RHS>(o, blk);
@@ -52,7 +55,6 @@ __device__ __forceinline__ void spec_pass(const SpecObj &o, int blk) {
   if (PASS == SP_BACK_FIRST) rows_back<DST_SET>(o, blk);
   if (PASS == SP_BACK) rows_back<DST_ADD>(o, blk);
   if (PASS == SP_BACK_LAST) rows_back<DST_ADD_LAST>(o, blk);
-  if (PASS == SP_CHECK) check(o, blk, o.check_blocks);
 }
 #ifndef IRTPS_COL_THREADS
 #define IRTPS_COL_THREADS 512
@@ -63,10 +65,100 @@ __global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) 
   spec_pass<PASS>(o, blockIdx.x);
 }
 
-// Batched: object i owns the blocks [blk[g] of i, blk[g] of i + 1) of a launch, g = 0 rows, 1 columns, 2 check.
-template <int PASS>
-__global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) k_spec_b(const SpecObj *__restrict__ objs, int n) {
-  constexpr int g = PASS == SP_COLS ? 1 : (PASS == SP_CHECK ? 2 : 0);
+// One more refinement step by the blocks of a cooperative launch (dynamic shared memory: one line pair).
+__device__ __noinline__ void refine_again(const SpecObj &o, Team t) {
+  CGCtl *ctl = o.ctl;
+  for (int i = t.bid; i < o.row_blocks; i += t.nblk) {
+    rows_forward<SRC_RESIDUAL>(o, i);
+    __syncthreads();
+  }
+  grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+  for (int i = t.bid; i < (o.W + 1) / 2; i += t.nblk) {
+    columns(o, i, 1);
+    __syncthreads();
+  }
+  grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+  for (int i = t.bid; i < o.row_blocks; i += t.nblk) {
+    rows_back<DST_ADD_LAST>(o, i);
+    __syncthreads();
+  }
+  grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+}
+
+// Sum of n partials by one warp, valid in its first lane.  (A warp's FP64 instruction holds the SM's FP64 pipe for 16
+// cycles: sums by one warp a block instead of all eight take 4 us off the last pass at 512 x 512.)
+__device__ __forceinline__ double warp_total(const double *part, int n) {
+  double v = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x & 31; i < n; i += 32) v += __ldcg(part + i);
+  for (int k = 16; k > 0; k >>= 1) v += __shfl_down_sync(0xffffffffu, v, k);
+  return v;
+}
+
+// The end of a solve (cooperative; 18 us at 512 x 512 and 25 at 637 x 899, where a plain launch whose last block
+// checks took 18 and 23): the FP64 residual against the tolerance, and the FP32 surface of mean zero (the
+// (0, 0) term was dropped, but FP32 transforms leave a mean of their rounding, which no residual sees).  While the
+// residual is above the tolerance and a step at least halves it, further refinement steps follow (a step lowers it
+// by orders of magnitude or has met the rounding of the FP64 residual).  Every block sums the same partials in the
+// same order and so takes the same decisions.
+constexpr int kMoreSteps = 8;
+__device__ __forceinline__ void finish(const SpecObj &o, Team t) {
+  __shared__ double s_sq[kSpecThreads], s_bb, s_mean, s_rel;
+  const int P = o.H * o.W, warp = threadIdx.x >> 5;
+  CGCtl *ctl = o.ctl;
+  double *part = o.part + 2 * o.row_blocks;
+  double rel, last = INFINITY;
+  for (int more = 0;; ++more) {
+    if (warp < 2) {
+      const double v = warp_total(o.part + warp * o.row_blocks, o.row_blocks);
+      if (threadIdx.x == 0) s_bb = v;
+      if (threadIdx.x == 32) s_mean = v * o.inv_p;
+    }
+    __syncthreads();
+    const double mean = s_mean;
+    double rr = 0.0;
+    for (int p = t.bid * blockDim.x + threadIdx.x; p < P; p += t.nblk * blockDim.x) {
+      const int i = p / o.W;
+      const double r = residual_at(o, i, p - i * o.W);
+      rr = fma(r, r, rr);
+      o.depth[p] = (float)(o.x[p] - mean);
+    }
+    s_sq[threadIdx.x] = rr;
+    __syncthreads();
+    if (warp == 0) {
+      for (int k = 1; k < kSpecThreads / 32; ++k) rr += s_sq[threadIdx.x + 32 * k];
+      for (int k = 16; k > 0; k >>= 1) rr += __shfl_down_sync(0xffffffffu, rr, k);
+      if (threadIdx.x == 0) part[t.bid] = rr;
+    }
+    grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
+    if (warp == 0) {
+      rr = warp_total(part, t.nblk);
+      if (threadIdx.x == 0) s_rel = s_bb > 0.0 ? sqrt(rr / s_bb) : 0.0;
+    }
+    __syncthreads();
+    rel = s_rel;
+    if (!(rel > o.tol) || !(rel < 0.5 * last) || more == kMoreSteps || *(volatile int *)&ctl->err) break;
+    last = rel;
+    refine_again(o, t);
+  }
+  if (t.bid == 0 && threadIdx.x == 0) {
+    ctl->rel = rel;
+    ctl->iters = 1;
+    o.acc->iters += 1;
+    o.acc->last_iters = 1;
+    o.acc->rel_last = rel;
+    if (*(volatile int *)&ctl->err) o.acc->err = 1;
+    if (!isfinite(s_bb) || !isfinite(rel) || rel > o.tol) o.acc->bad = 1;
+  }
+}
+
+// The last pass, cooperative (registers for the four blocks an SM that the residual's loads want).
+__global__ void __launch_bounds__(kSpecThreads, 4) k_spec_finish(const __grid_constant__ SpecObj o) {
+  finish(o, Team{(int)blockIdx.x, (int)gridDim.x});
+}
+
+// Batched: object i owns the blocks [blk[g] of i, blk[g] of i + 1) of a launch, g = 0 rows, 1 columns, 2 last pass.
+__device__ __forceinline__ int object_of(const SpecObj *__restrict__ objs, int n, int g) {
   __shared__ int s_o;
   if (threadIdx.x == 0) {
     int lo = 0, hi = n - 1;
@@ -77,8 +169,17 @@ __global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) 
     s_o = lo;
   }
   __syncthreads();
-  const SpecObj &o = objs[s_o];
+  return s_o;
+}
+template <int PASS>
+__global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) k_spec_b(const SpecObj *__restrict__ objs, int n) {
+  constexpr int g = PASS == SP_COLS ? 1 : 0;
+  const SpecObj &o = objs[object_of(objs, n, g)];
   spec_pass<PASS>(o, (int)blockIdx.x - o.blk[g]);
+}
+__global__ void __launch_bounds__(kSpecThreads, 4) k_spec_finish_b(const SpecObj *__restrict__ objs, int n) {
+  const SpecObj &o = objs[object_of(objs, n, 2)];
+  finish(o, Team{(int)blockIdx.x - o.blk[2], o.check_blocks});
 }
 
 // ---- host: plans ----
@@ -169,9 +270,22 @@ PlanTables make_plan(int n, std::vector<float2> &pool) {
 size_t row_smem(const SpecObj &o) { return sizeof(float2) * 2 * line_stride(o.row.m); }
 size_t col_smem(const SpecObj &o) { return sizeof(float2) * 2 * o.col_lines * line_stride(o.col.m); }
 
-// Refinement steps after the first solve: two pass the default tolerance (1e-9) with two orders of margin on
-// every grid up to 4096 on a side, and one does up to 128 on a side (residual 5e-12 at 64, 3e-11 at 129); tighter
-// tolerances get four, down to the floor of FP64.
+size_t line_smem(const FftPlan &row, const FftPlan &col) {
+  return sizeof(float2) * 2 * (size_t)std::max(line_stride(row.m), line_stride(col.m));
+}
+// Co-resident blocks of the last pass (also raises its shared-memory limit); 0 on an error.
+template <typename F>
+int finish_blocks_most(F *k, size_t smem, int sms) {
+  int per = 0;
+  if (allow_max_smem((const void *)k) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kSpecThreads, smem) != cudaSuccess)
+    return 0;
+  return std::min(per, 4) * (sms > 0 ? sms : 1);
+}
+
+// Refinement steps launched ahead of the last pass, which adds those that are missing at one pass's speed of a
+// cooperative grid: one up to 128 on a side (residual 2e-10 or less at the default tolerance of 1e-9), two beyond
+// (4e-10 or less to 2048; from there on smooth slopes take a third), four for tolerances near the floor of FP64.
 int refinements(const SpecObj &o) { return o.tol < 1e-10 ? 4 : (std::max(o.H, o.W) <= 128 ? 1 : 2); }
 
 }  // namespace
@@ -199,7 +313,6 @@ cudaError_t spectral_setup(Ctx &c) {
   o.H = H;
   o.W = W;
   o.row_blocks = (H + 1) / 2;
-  o.check_blocks = std::min((H * W + kSpecThreads - 1) / kSpecThreads, 4 * (c.sms > 0 ? c.sms : 1));
   // column lines per block: the widest loads (8 columns, a 32-byte sector) that still give every SM a block
   o.col_lines = 1;
   for (int L : {4, 2})
@@ -208,13 +321,16 @@ cudaError_t spectral_setup(Ctx &c) {
       o.col_lines = L;
   o.col_blocks = (W + 2 * o.col_lines - 1) / (2 * o.col_lines);
   const size_t pb = sizeof(float2) * pool.size(), lb = (sizeof(float) * lam.size() + 15) / 16 * 16;
-  const size_t qb = sizeof(double) * (2 * o.row_blocks + o.check_blocks);
   cudaError_t e = cudaSuccess;
   for (const void *k : {(const void *)k_spec<SP_ROWS_FIRST>, (const void *)k_spec<SP_ROWS>, (const void *)k_spec<SP_COLS>,
                         (const void *)k_spec<SP_BACK_FIRST>, (const void *)k_spec<SP_BACK>,
                         (const void *)k_spec<SP_BACK_LAST>})
     if ((e = allow_max_smem(k)) != cudaSuccess) return e;
   if (c.opt.irls_iters > 0 && (e = cg_allow_smem()) != cudaSuccess) return e;
+  const int most = finish_blocks_most(k_spec_finish, line_smem(row.p, col.p), c.sms);
+  if (most < 1) return cudaErrorInvalidConfiguration;
+  o.check_blocks = std::min((H * W + kSpecThreads - 1) / kSpecThreads, most);
+  const size_t qb = sizeof(double) * (2 * o.row_blocks + o.check_blocks);
   e = cudaMalloc(&c.sp_pool, pb + lb + qb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c.sp_t, sizeof(float) * (size_t)H * W);
   if (e != cudaSuccess) return e;
@@ -255,9 +371,7 @@ SpecObj spec_object(const Ctx &c, CGAcc *acc) {
   return o;
 }
 
-size_t spec_line_smem(const Ctx &c) {
-  return sizeof(float2) * 2 * (size_t)std::max(line_stride(c.sp.row.m), line_stride(c.sp.col.m));
-}
+size_t spec_line_smem(const Ctx &c) { return line_smem(c.sp.row, c.sp.col); }
 
 cudaError_t launch_spectral(Ctx &c) {
   const SpecObj o = spec_object(c, &c.dstats->cg);
@@ -275,7 +389,10 @@ cudaError_t launch_spectral(Ctx &c) {
     else
       k_spec<SP_BACK_LAST><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
   }
-  k_spec<SP_CHECK><<<o.check_blocks, kSpecThreads, 0, s>>>(o);
+  void *args[] = {(void *)&o};
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_spec_finish, dim3(o.check_blocks),
+                                                    dim3(kSpecThreads), args, line_smem(o.row, o.col), s);
+  if (e != cudaSuccess) return e;
   c.stats.launches += 4 + 3 * n;
   return cudaGetLastError();
 }
@@ -290,12 +407,11 @@ cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, S
     SpecObj o = spec_object(c, &ds[i].cg);
     o.blk[0] = sb.blocks[0];
     o.blk[1] = sb.blocks[1];
-    o.blk[2] = sb.blocks[2];
     sb.blocks[0] += o.row_blocks;
     sb.blocks[1] += o.col_blocks;
-    sb.blocks[2] += o.check_blocks;
     sb.row_smem = std::max(sb.row_smem, row_smem(o));
     sb.col_smem = std::max(sb.col_smem, col_smem(o));
+    sb.line_smem = std::max(sb.line_smem, line_smem(o.row, o.col));
     sb.refine = std::max(sb.refine, refinements(o));
     t.push_back(o);
     ++sb.n;
@@ -306,6 +422,17 @@ cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, S
                         (const void *)k_spec_b<SP_COLS>, (const void *)k_spec_b<SP_BACK_FIRST>,
                         (const void *)k_spec_b<SP_BACK>, (const void *)k_spec_b<SP_BACK_LAST>})
     if ((e = allow_max_smem(k)) != cudaSuccess) return e;
+  // last pass: the co-resident blocks shared in proportion to the pixel counts, at least one an object
+  const int most = finish_blocks_most(k_spec_finish_b, sb.line_smem, objs[0]->sms);
+  if (most < sb.n) return cudaErrorInvalidConfiguration;
+  double pixels = 0.0;
+  for (const SpecObj &o : t) pixels += (double)o.H * o.W;
+  for (SpecObj &o : t) {
+    const int share = 1 + (int)((double)(most - sb.n) * ((double)o.H * o.W) / pixels);
+    o.check_blocks = std::min(o.check_blocks, share);
+    o.blk[2] = sb.blocks[2];
+    sb.blocks[2] += o.check_blocks;
+  }
   e = cudaMalloc(&sb.table, sizeof(SpecObj) * sb.n);
   if (e != cudaSuccess) return e;
   return cudaMemcpy(sb.table, t.data(), sizeof(SpecObj) * sb.n, cudaMemcpyHostToDevice);
@@ -329,7 +456,10 @@ cudaError_t launch_spectral_batch(cudaStream_t s, const SpectralBatch &sb) {
     else
       k_spec_b<SP_BACK_LAST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
   }
-  k_spec_b<SP_CHECK><<<sb.blocks[2], kSpecThreads, 0, s>>>(t, n);
+  void *args[] = {(void *)&t, (void *)&n};
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_spec_finish_b, dim3(sb.blocks[2]),
+                                                    dim3(kSpecThreads), args, sb.line_smem, s);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

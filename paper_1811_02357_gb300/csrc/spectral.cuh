@@ -316,7 +316,10 @@ __device__ __forceinline__ void rows_forward(const SpecObj &o, int blk, F load =
     bb = block_sum(bb, sh);
     if (threadIdx.x == 0) {
       o.part[blk] = bb;
-      if (blk == 0) o.ctl->count = 0u;  // arrivals of the check pass
+      if (blk == 0) {  // barrier state of the last pass
+        o.ctl->count = 0u;
+        o.ctl->err = 0;
+      }
     }
   }
   const float2 *z = dft_lines(P, a, b, 1);
@@ -417,57 +420,6 @@ __device__ __forceinline__ void rows_back(const SpecObj &o, int blk, F store = F
     __shared__ double sh[32];
     sum = block_sum(sum, sh);
     if (threadIdx.x == 0) o.part[o.row_blocks + blk] = sum;
-  }
-}
-
-// The FP64 residual against the tolerance, and the FP32 surface of mean zero (the (0, 0) term was dropped, but
-// FP32 transforms leave a mean of their rounding, which no residual sees).
-__device__ __forceinline__ void check(const SpecObj &o, int blk, int nblk) {
-  __shared__ double sh[32];
-  __shared__ double s_mean;
-  __shared__ bool last;
-  const int P = o.H * o.W;
-  double rr = 0.0;
-  for (int i = threadIdx.x; i < o.row_blocks; i += blockDim.x) rr += __ldcg(o.part + o.row_blocks + i);
-  rr = block_sum(rr, sh);
-  if (threadIdx.x == 0) s_mean = rr * o.inv_p;
-  __syncthreads();
-  const double mean = s_mean;
-  float rf = 0.0f;
-  for (int p = blk * blockDim.x + threadIdx.x; p < P; p += nblk * blockDim.x) {
-    const int i = p / o.W;
-    // FP32 squares (a thread's few dozen), scaled clear of underflow: the FP64 pipe bounds this pass
-    const float r = (float)residual_at(o, i, p - i * o.W) * 1.099511627776e12f;  // 2^40
-    rf = fmaf(r, r, rf);
-    o.depth[p] = (float)(o.x[p] - mean);
-  }
-  rr = block_sum((double)rf * 8.271806125530277e-25, sh);  // 2^-80
-  double *part = o.part + 2 * o.row_blocks;
-  if (threadIdx.x == 0) {
-    part[blk] = rr;
-    __threadfence();
-    last = atomicAdd(&o.ctl->count, 1u) == (unsigned)nblk - 1u;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double bb = 0.0;
-  rr = 0.0;
-  for (int i = threadIdx.x; i < o.row_blocks; i += blockDim.x) bb += __ldcg(o.part + i);
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x) rr += __ldcg(part + i);
-  bb = block_sum(bb, sh);
-  __syncthreads();
-  rr = block_sum(rr, sh);
-  if (threadIdx.x == 0) {
-    CGCtl *ctl = o.ctl;
-    // one FP64 division and a FP32 root: a chain of FP64 roots by one thread takes longer than the pass itself
-    ctl->count = 0u;
-    ctl->rel = bb > 0.0 ? (double)sqrtf((float)(rr / bb)) : 0.0;
-    ctl->iters = 1;
-    o.acc->iters += 1;
-    o.acc->last_iters = 1;
-    o.acc->rel_last = ctl->rel;
-    if (!isfinite(bb) || !isfinite(ctl->rel) || ctl->rel > o.tol) o.acc->bad = 1;
   }
 }
 
