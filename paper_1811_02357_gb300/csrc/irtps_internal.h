@@ -110,6 +110,7 @@ struct SpecObj {
   FftPlan row, col;      // lengths W and H
   const float *mu, *nu;  // eigenvalues of the columns' and rows' path Laplacians
   int row_blocks, col_blocks, check_blocks;
+  int refine;            // refinement steps launched ahead of the last pass
   int col_lines;         // complex lines (pairs of columns) per block of the column pass
   int blk[3];            // first block in a batched launch: row, column, last passes
 };
@@ -283,7 +284,7 @@ inline bool direct_solve(const Ctx &c) { return c.opt.precond == 2 && c.sp_t != 
 struct SpectralBatch {
   int n = 0;              // objects with direct solves
   int blocks[3] = {0};    // row, column, last passes
-  int refine = 0;         // refinement steps
+  int refine = 0;         // most refinement steps of an object
   size_t row_smem = 0, col_smem = 0, line_smem = 0;
   void *table = nullptr;  // owned
 };

@@ -171,11 +171,17 @@ __device__ __forceinline__ int object_of(const SpecObj *__restrict__ objs, int n
   __syncthreads();
   return s_o;
 }
+// step: -1 for the first solve, then the refinement steps; an object takes as many as it does alone.
 template <int PASS>
-__global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) k_spec_b(const SpecObj *__restrict__ objs, int n) {
+__global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads)
+    k_spec_b(const SpecObj *__restrict__ objs, int n, int step) {
   constexpr int g = PASS == SP_COLS ? 1 : 0;
   const SpecObj &o = objs[object_of(objs, n, g)];
-  spec_pass<PASS>(o, (int)blockIdx.x - o.blk[g]);
+  if (step >= o.refine) return;
+  if (PASS == SP_BACK && step + 1 == o.refine)
+    spec_pass<SP_BACK_LAST>(o, (int)blockIdx.x - o.blk[g]);
+  else
+    spec_pass<PASS>(o, (int)blockIdx.x - o.blk[g]);
 }
 __global__ void __launch_bounds__(kSpecThreads, 4) k_spec_finish_b(const SpecObj *__restrict__ objs, int n) {
   const SpecObj &o = objs[object_of(objs, n, 2)];
@@ -286,7 +292,7 @@ int finish_blocks_most(F *k, size_t smem, int sms) {
 // Refinement steps launched ahead of the last pass, which adds those that are missing at one pass's speed of a
 // cooperative grid: one up to 128 on a side (residual 2e-10 or less at the default tolerance of 1e-9), two beyond
 // (4e-10 or less to 2048; from there on smooth slopes take a third), four for tolerances near the floor of FP64.
-int refinements(const SpecObj &o) { return o.tol < 1e-10 ? 4 : (std::max(o.H, o.W) <= 128 ? 1 : 2); }
+int refinements(const Ctx &c) { return c.opt.cg_tol < 1e-10 ? 4 : (std::max(c.H, c.W) <= 128 ? 1 : 2); }
 
 }  // namespace
 
@@ -362,6 +368,7 @@ SpecObj spec_object(const Ctx &c, CGAcc *acc) {
   o.inv_p = 1.0 / ((double)c.H * c.W);
   o.nz_min = c.opt.nz_min;
   o.tol = c.opt.cg_tol;
+  o.refine = refinements(c);
   o.nrm = c.nrm;
   o.depth = c.depth;
   o.x = c.cg_x;
@@ -380,7 +387,7 @@ cudaError_t launch_spectral(Ctx &c) {
   k_spec<SP_ROWS_FIRST><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
   k_spec<SP_COLS><<<o.col_blocks, kColThreads, cs, s>>>(o);
   k_spec<SP_BACK_FIRST><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
-  const int n = refinements(o);
+  const int n = o.refine;
   for (int i = 0; i < n; ++i) {
     k_spec<SP_ROWS><<<o.row_blocks, kSpecThreads, rs, s>>>(o);
     k_spec<SP_COLS><<<o.col_blocks, kColThreads, cs, s>>>(o);
@@ -412,7 +419,7 @@ cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, S
     sb.row_smem = std::max(sb.row_smem, row_smem(o));
     sb.col_smem = std::max(sb.col_smem, col_smem(o));
     sb.line_smem = std::max(sb.line_smem, line_smem(o.row, o.col));
-    sb.refine = std::max(sb.refine, refinements(o));
+    sb.refine = std::max(sb.refine, o.refine);
     t.push_back(o);
     ++sb.n;
   }
@@ -420,7 +427,7 @@ cudaError_t spectral_batch_setup(const std::vector<Ctx *> &objs, DevStats *ds, S
   cudaError_t e = cudaSuccess;
   for (const void *k : {(const void *)k_spec_b<SP_ROWS_FIRST>, (const void *)k_spec_b<SP_ROWS>,
                         (const void *)k_spec_b<SP_COLS>, (const void *)k_spec_b<SP_BACK_FIRST>,
-                        (const void *)k_spec_b<SP_BACK>, (const void *)k_spec_b<SP_BACK_LAST>})
+                        (const void *)k_spec_b<SP_BACK>})
     if ((e = allow_max_smem(k)) != cudaSuccess) return e;
   // last pass: the co-resident blocks shared in proportion to the pixel counts, at least one an object
   const int most = finish_blocks_most(k_spec_finish_b, sb.line_smem, objs[0]->sms);
@@ -445,16 +452,13 @@ cudaError_t launch_spectral_batch(cudaStream_t s, const SpectralBatch &sb) {
   const SpecObj *t = (const SpecObj *)sb.table;
   const int n = sb.n;
   const size_t rs = sb.row_smem, cs = sb.col_smem;
-  k_spec_b<SP_ROWS_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
-  k_spec_b<SP_COLS><<<sb.blocks[1], kColThreads, cs, s>>>(t, n);
-  k_spec_b<SP_BACK_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
+  k_spec_b<SP_ROWS_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n, -1);
+  k_spec_b<SP_COLS><<<sb.blocks[1], kColThreads, cs, s>>>(t, n, -1);
+  k_spec_b<SP_BACK_FIRST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n, -1);
   for (int i = 0; i < sb.refine; ++i) {
-    k_spec_b<SP_ROWS><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
-    k_spec_b<SP_COLS><<<sb.blocks[1], kColThreads, cs, s>>>(t, n);
-    if (i + 1 < sb.refine)
-      k_spec_b<SP_BACK><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
-    else
-      k_spec_b<SP_BACK_LAST><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n);
+    k_spec_b<SP_ROWS><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n, i);
+    k_spec_b<SP_COLS><<<sb.blocks[1], kColThreads, cs, s>>>(t, n, i);
+    k_spec_b<SP_BACK><<<sb.blocks[0], kSpecThreads, rs, s>>>(t, n, i);
   }
   void *args[] = {(void *)&t, (void *)&n};
   const cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_spec_finish_b, dim3(sb.blocks[2]),
