@@ -102,8 +102,10 @@ __device__ __forceinline__ float norm_zxy(float x, float y, float z) {
 
 // Normal and albedo of pixel p from G (Eq. 4 and the text after it): n = normalize(sum_c G_c),
 // rho_c = |G_c|; a pixel whose solve failed (ok false) or whose sum vanishes is invalid.
-template <int C, bool LISTED = false>
-__device__ __forceinline__ void ps_store(const PSArgs &a, int p, const float (&G)[3][C], bool ok) {
+// `listed`: G comes from ps_masked_fp64, whose one-channel albedo is the norm that scales the normal (the other solves'
+// is summed in the other order); in every form of the kernel, so that a pixel's bits do not depend on the form.
+template <int C>
+__device__ __forceinline__ void ps_store(const PSArgs &a, int p, const float (&G)[3][C], bool ok, bool listed = false) {
   const size_t P = (size_t)a.P;
   float sx = 0.0f, sy = 0.0f, sz = 0.0f;
 #pragma unroll
@@ -119,7 +121,7 @@ __device__ __forceinline__ void ps_store(const PSArgs &a, int p, const float (&G
   float rout[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    rout[c] = !ok ? 0.0f : (C == 1 && LISTED) ? norm : norm_zxy(G[0][c], G[1][c], G[2][c]);
+    rout[c] = !ok ? 0.0f : (C == 1 && listed) ? norm : norm_zxy(G[0][c], G[1][c], G[2][c]);
     rsum += rout[c];
   }
   if (ok) {
@@ -374,10 +376,10 @@ __device__ __forceinline__ bool ps_masked_fp64(const PSArgs &a, int p, const flo
 
 template <int C, typename TI>
 __device__ __forceinline__ bool ps_masked_solve(const PSArgs &a, int p, const float (&R)[3][C], float (&G)[3][C],
-                                                unsigned long long valid) {
+                                                unsigned long long valid, bool &listed) {
   const int st = ps_masked_fp32<C>(a, R, G, valid);
-  if (st != PS_NEED_FP64) return st == PS_SOLVED;
-  return ps_masked_fp64<C, TI>(a, p, R, G, valid);
+  listed = st == PS_NEED_FP64;
+  return listed ? ps_masked_fp64<C, TI>(a, p, R, G, valid) : st == PS_SOLVED;
 }
 
 // The rest of pixel p once every row is in: the masked solve when some row is masked
@@ -387,10 +389,10 @@ template <int C, typename TI, bool NE>
 __device__ __forceinline__ void ps_finish(const PSArgs &a, int p, const float (&R)[3][C], float (&G)[3][C],
                                           unsigned long long valid) {
   const unsigned long long all = a.K == 64 ? ~0ull : ((1ull << a.K) - 1ull);
-  bool ok = true;
-  if (valid != all) ok = ps_masked_solve<C, TI>(a, p, R, G, valid);
+  bool ok = true, listed = false;
+  if (valid != all) ok = ps_masked_solve<C, TI>(a, p, R, G, valid, listed);
   else if (NE) ps_apply_minv<C>(a, R, G);
-  ps_store<C>(a, p, G, ok);
+  ps_store<C>(a, p, G, ok, listed);
 }
 
 template <int C, typename TI, bool NE>
@@ -612,7 +614,7 @@ __global__ void __launch_bounds__(128, kPsMaskedBlocks) k_ps_masked(const PSArgs
 #pragma unroll
       for (int c = 0; c < C; ++c) R[r][c] = L.rhs[(size_t)i * 9 + r * C + c];
     const bool ok = ps_masked_fp64<C, TI>(a, p, R, G, L.mask[i]);
-    ps_store<C, true>(a, p, G, ok);
+    ps_store<C>(a, p, G, ok, true);
   }
 }
 
