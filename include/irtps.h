@@ -64,7 +64,7 @@ typedef struct irtps_options {
   double cond_max;    /* masked 3x3 solves with 1-norm condition above this: invalid pixel (1e8) */
   float nz_min;       /* n_z clamp of the slopes -n_x/n_z, -n_y/n_z (0.05) */
   double cg_tol;      /* depth solve: stop at FP64 |b - A x| / |b| <= cg_tol (1e-9) */
-  int cg_max_iter;    /* depth solve iteration cap (50000) */
+  int cg_max_iter;    /* depth solve iteration cap, of each preconditioner where a solve changes it (50000) */
   int cg_check_every; /* FP64 true-residual refresh and convergence test period (10) */
   double stop_tol;    /* irtps_iterate stops early when D_H < stop_tol; 0 = never (0) */
   int precond;        /* depth solve: 0 Jacobi-preconditioned CG, 1 multigrid-preconditioned CG,
@@ -72,7 +72,8 @@ typedef struct irtps_options {
                          transform that diagonalises the grid Laplacian (fast transforms in FP32,
                          refined until the FP64 residual is within cg_tol or falls no further; one
                          iteration in the statistics),
-                         which also preconditions their weighted (irls) solves; larger grids use
+                         which also preconditions their weighted (irls) solves while that is expected to
+                         be the faster way (else they go over to multigrid); larger grids use
                          multigrid (2) */
   int use_graph;      /* 1: irtps_iterate captures one iteration as a CUDA graph and replays it (0);
                          per-stage times are then not measured (reported as 0) */

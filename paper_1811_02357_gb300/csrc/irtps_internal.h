@@ -111,6 +111,7 @@ struct SpecObj {
   const float *mu, *nu;  // eigenvalues of the columns' and rows' path Laplacians
   int row_blocks, col_blocks, check_blocks;
   int refine;            // refinement steps launched ahead of the last pass
+  int limit;             // weighted solves: iterations beyond which multigrid is the faster preconditioner
   int col_lines;         // complex lines (pairs of columns) per block of the column pass
   int blk[3];            // first block in a batched launch: row, column, last passes
 };
@@ -276,6 +277,7 @@ SpecObj spec_object(const Ctx &c, CGAcc *acc);
 // belongs to the function and not to a context, so it is set to this one value wherever it is set: a size of the
 // caller's own would refuse the launches of other threads' contexts that take more.
 cudaError_t allow_max_smem(const void *kernel);
+int spectral_limit(const Ctx &c, int nblk);
 size_t spec_line_smem(const Ctx &c);  // shared memory of one line pair, rows or columns
 cudaError_t launch_spectral(Ctx &c);  // the whole solve: normals -> b, x, depth, residual check
 // whether a context's unit-weight solves are direct (option precond = 2 on a grid the transform covers)

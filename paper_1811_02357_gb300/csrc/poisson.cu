@@ -441,9 +441,11 @@ __device__ void mg_vcycle(const MG &m, const float *r, CGCtl *ctl, Team t) {
 #undef MG_FOR
 
 // z = A_1^+ r by the FP32 cosine transforms (A_1 the unit-weight Laplacian), a preconditioner of the weighted
-// solves: the Huber weights lie in (0, 1] and differ from 1 at a tenth of the edges, so PCG takes 16 to 21
-// iterations to 1e-9 whatever the grid, where the V-cycle takes some thirty barriers and several times the
-// iterations.  With `update` the step comes first, e += af p, r -= af Ap: a block transforms the rows that it
+// solves.  The Huber weights lie in (0, 1]; where few of them are far below 1, PCG takes 16 to 40 iterations to 1e-9
+// whatever the grid, of a third to a half of the time of the V-cycle's, which takes some thirty barriers.  With outliers
+// or a small threshold the weights spread over orders of magnitude, which this preconditioner does not follow (5 %
+// outliers, threshold 0.05: 80 to 90 iterations, 1e-3: 470, 1e-4: 1200; the V-cycle 70 to 260): the solve then
+// goes over to the V-cycle (Follow).  With `update` the step comes first, e += af p, r -= af Ap: a block transforms the rows that it
 // updates, which saves a pass and a barrier.  Returns the thread's sums of r.z and (with `update`) of (rscale r)^2.
 // Two barriers; the caller's next one publishes z.  One copy in the code (the FFT stages are long).
 // With the step inside, no solve for a residual about to be refreshed, and the refresh by the FP32 residual, classic PS
@@ -497,16 +499,50 @@ __device__ __noinline__ float2 spectral_solve(const SpecObj &o, const CG &g, flo
 // refreshes when the FP32 residual falls below tol / 2, since its iterations are few and dear.
 // Dot products are FP32 within a block and FP64 across blocks; every block sums the same partials in the same
 // order and so takes the same decisions.
+//
+// A PRE 2 solve that is expected to take more than so->limit iterations (Follow), or has taken max_iter, returns
+// early (`change`) for the caller to go on with PRE 1 from its iterate, by max_iter iterations at most: an iteration
+// cap that the V-cycle by itself stays below is then enough.
+struct Progress {
+  int it = 0;         // iterations so far
+  double rel = 0.0;   // FP64 relative residual (it > 0)
+  bool change = false;
+};
+
+// The course of a spectral solve: from the largest residual met (CG's rises at first) and the lowest since, in units of
+// the tolerance, the iterations that it will take at this rate.
+struct Follow {
+  float peak, low;
+  int peak_it = 0;
+  __device__ __forceinline__ explicit Follow(float ratio) : peak(ratio), low(ratio) {}
+  __device__ __forceinline__ void at(int it, float ratio) {
+    if (ratio > peak) {
+      peak = low = ratio;
+      peak_it = it;
+    } else {
+      low = fminf(low, ratio);
+    }
+  }
+  // Looked at from an eighth of the limit on; at the limit itself the solve goes over unless it is done.
+  __device__ __forceinline__ bool too_slow(int it, int limit) const {
+    if (!(low > 1.0f)) return false;
+    if (it >= limit) return true;
+    const int n = it - peak_it;
+    return 8 * n >= limit && n >= 4 && (float)n * __logf(low) > (float)(limit - it) * __logf(peak / low);
+  }
+};
+
 template <int PRE, bool WEIGHTED>
-__device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc, double tol, int max_iter, int check,
-                                             const MG &mg, const SpecObj *so, Team t) {
+__device__ __forceinline__ Progress cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc, double tol, int max_iter,
+                                                 int check, const MG &mg, const SpecObj *so, Team t,
+                                                 Progress start = Progress()) {
   __shared__ double sh[33];
   __shared__ float shf[33];
   __shared__ float s_ab[2];
-  __shared__ int s_frozen;
+  __shared__ int s_frozen, s_slow;
   double best = INFINITY;
   int stall = 0, it = 0;
-  double rel = ctl->rel;
+  double rel = start.it > 0 ? start.rel : ctl->rel;
   const double bnorm = ctl->bnorm;
   if (!(bnorm > 0.0) || !isfinite(bnorm)) rel = 0.0;  // flat (or broken) right-hand side: nothing to solve
   float *e = g.ap + g.P;  // correction accumulator (second half of the Ap buffer)
@@ -543,9 +579,10 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
       if (threadIdx.x == 0) g.part[S_RS * g.stride + t.bid] = (double)rs;
     }
   };
+  Follow follow((float)(rel / tol));  // (thread 0's counts)
   // Refresh from FP64: x64 += e, e = 0, r = b - A x64, its norm against tol, and z, r.z of iteration `it` unless the
-  // solve ends here (returned).  `af`: the step along p that e still lacks.
-  auto refresh = [&](float af, const float *p) -> bool {
+  // solve ends here (returned) or `go_on` is false.  `af`: the step along p that e still lacks.
+  auto refresh = [&](float af, const float *p, bool go_on = true) -> bool {
     for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) {
       g.x[q.p] += (double)fmaf(af, p[q.p], e[q.p]);
       e[q.p] = 0.0f;
@@ -567,6 +604,8 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
     if (*(volatile int *)&ctl->err) return true;
     rel = sqrt(total(g.part + S_RR * g.stride, g.nblk, sh)) / bnorm;
     if (!isfinite(rel) || !(rel > tol)) return true;
+    if (!go_on) return false;
+    if (PRE == 2 && threadIdx.x == 0) follow.at(it, (float)(rel / tol));
     if (rel < 0.95 * best) {
       best = rel;
       stall = it;
@@ -584,12 +623,14 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
   }
   double num = 0.0, ref = 0.0;  // r.z of the last iteration and of the last refresh
   int fresh = 0;                // the iteration of the last refresh
+  bool change = false;
   while (rel > tol && it < max_iter && !*(volatile int *)&ctl->err) {
     // ---- A ----
     const double den = num;
     if (PRE == 2 && it >= fresh + 3) {  // refresh once the FP32 residual says that the solve is done
       const double2 s = total2(g.part + (S_RZ0 + (it & 1)) * g.stride, g.part + S_RS * g.stride, g.nblk, sh);
       num = s.x;
+      if (threadIdx.x == 0) follow.at(it, sqrtf((float)s.y));
       if (s.y <= 0.25) {
         fresh = it;
         if (refresh(0.0f, e)) break;
@@ -603,9 +644,15 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
     if (threadIdx.x == 0) {
       const bool frozen = !(num > 1e-10 * ref);
       s_frozen = frozen;
+      if (PRE == 2) s_slow = follow.too_slow(it - 1, so->limit);
       s_ab[1] = (it > 1 && !frozen && den > 0.0) ? (float)(num / den) : 0.0f;
     }
     __syncthreads();
+    if (PRE == 2 && s_slow) {
+      --it;
+      change = true;
+      break;
+    }
     const bool frozen = s_frozen;
     const float beta = s_ab[1];
     const bool first = it == 1;
@@ -659,18 +706,49 @@ __device__ __forceinline__ void cg_loop_body(const CG &g, CGCtl *ctl, CGAcc *acc
     grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
     if (*(volatile int *)&ctl->err) break;
   }
+  if (PRE == 2 && (change || (it == max_iter && it > 0)) && rel > tol && isfinite(rel) && !*(volatile int *)&ctl->err) {
+    change = !refresh(0.0f, e, false);  // r for the next preconditioner, if the solve isn't done
+    if (change) return Progress{it, rel, true};
+  }
   // fold in a correction collected since the last refresh (none when the loop ended on a refresh)
   for (Stride q(g.W, t); q.p < g.P; q.next(g.W)) g.x[q.p] += (double)e[q.p];
   if (t.bid == 0 && threadIdx.x == 0) {
-    ctl->iters = it;
+    ctl->iters = start.it + it;
     ctl->rel = rel;
     if (acc) {
-      acc->iters += it;
-      acc->last_iters = it;
+      acc->iters += start.it + it;
+      acc->last_iters = start.it + it;
       acc->rel_last = rel;
       if (*(volatile int *)&ctl->err) acc->err = 1;
       if (!isfinite(bnorm) || !isfinite(rel) || rel > tol) acc->bad = 1;
     }
+  }
+  return Progress{start.it + it, rel, false};
+}
+
+// Galerkin weights of level l+1 from level l (2x2 aggregates): the sum of the fine
+// edge weights crossing between two aggregates (the host's construction, on the device).
+__device__ __forceinline__ void mg_coarsen_body(const MG &m, int l, float *wh, float *wv, Team t) {
+  const int Hf = m.H[l], Wf = m.W[l], Hc = m.H[l + 1], Wc = m.W[l + 1];
+  const float *fh = wh + m.off[l], *fv = wv + m.off[l];
+  float *ch = wh + m.off[l + 1], *cv = wv + m.off[l + 1];
+  for (int q = t.bid * blockDim.x + threadIdx.x; q < Hc * Wc; q += t.nblk * blockDim.x) {
+    const int I = q / Wc, J = q - I * Wc;
+    float sh = 0.0f, sv = 0.0f;
+    if (2 * J + 2 < Wf)
+      for (int i = 2 * I; i < 2 * I + 2 && i < Hf; ++i) sh += fh[i * Wf + 2 * J + 1];
+    if (2 * I + 2 < Hf)
+      for (int j = 2 * J; j < 2 * J + 2 && j < Wf; ++j) sv += fv[(2 * I + 1) * Wf + j];
+    ch[q] = sh;
+    cv[q] = sv;
+  }
+}
+
+// The whole hierarchy, by the blocks of a cooperative launch.
+__device__ __forceinline__ void mg_coarsen_all(const MG &m, float *wh, float *wv, CGCtl *ctl, Team t) {
+  for (int l = 0; l + 1 < m.levels; ++l) {
+    mg_coarsen_body(m, l, wh, wv, t);
+    grid_barrier(&ctl->count, &ctl->gen, &ctl->err, t.nblk);
   }
 }
 
@@ -680,10 +758,17 @@ __global__ void __launch_bounds__(kThreads) k_cg_loop(const CG g, CGCtl *ctl, CG
   cg_loop_body<PRE, WEIGHTED>(g, ctl, acc, tol, max_iter, check, mg, nullptr, whole_grid());
 }
 __global__ void __launch_bounds__(kThreads) k_cg_loop_spectral(const CG g, CGCtl *ctl, CGAcc *acc, double tol,
-                                                               int max_iter, int check,
+                                                               int max_iter, int check, const __grid_constant__ MG mg,
+                                                               float *wh, float *wv,
                                                                const __grid_constant__ SpecObj so) {
-  const MG none{};
-  cg_loop_body<2, true>(g, ctl, acc, tol, max_iter, check, none, &so, whole_grid());
+  const Team t = whole_grid();
+  Progress p;
+  if (so.limit > 0) {
+    p = cg_loop_body<2, true>(g, ctl, acc, tol, max_iter, check, mg, &so, t);
+    if (!p.change) return;
+  }
+  mg_coarsen_all(mg, wh, wv, ctl, t);
+  cg_loop_body<1, true>(g, ctl, acc, tol, max_iter, check, mg, nullptr, t, p);
 }
 static_assert(kThreads == spec::kSpecThreads, "the spectral passes run in the solver's blocks");
 
@@ -918,24 +1003,6 @@ __device__ __forceinline__ void irls_weights_body(const CG &g, float *wh, float 
   }
 }
 
-// Galerkin weights of level l+1 from level l (2x2 aggregates): the sum of the fine
-// edge weights crossing between two aggregates (the host's construction, on the device).
-__device__ __forceinline__ void mg_coarsen_body(const MG &m, int l, float *wh, float *wv, Team t) {
-  const int Hf = m.H[l], Wf = m.W[l], Hc = m.H[l + 1], Wc = m.W[l + 1];
-  const float *fh = wh + m.off[l], *fv = wv + m.off[l];
-  float *ch = wh + m.off[l + 1], *cv = wv + m.off[l + 1];
-  for (int q = t.bid * blockDim.x + threadIdx.x; q < Hc * Wc; q += t.nblk * blockDim.x) {
-    const int I = q / Wc, J = q - I * Wc;
-    float sh = 0.0f, sv = 0.0f;
-    if (2 * J + 2 < Wf)
-      for (int i = 2 * I; i < 2 * I + 2 && i < Hf; ++i) sh += fh[i * Wf + 2 * J + 1];
-    if (2 * I + 2 < Hf)
-      for (int j = 2 * J; j < 2 * J + 2 && j < Wf; ++j) sv += fv[(2 * I + 1) * Wf + j];
-    ch[q] = sh;
-    cv[q] = sv;
-  }
-}
-
 __global__ void __launch_bounds__(kThreads) k_irls_weights(const CG g, float *wh, float *wv, double delta) {
   irls_weights_body(g, wh, wv, delta, whole_grid());
 }
@@ -974,9 +1041,11 @@ static cudaError_t solve_once(Ctx &c) {
   MG mg = make_mg(c);
   if (WEIGHTED) mg.cscale = 1.0f;
   SpecObj so = spectral ? spec_object(c, acc) : SpecObj{};
-  void *args[] = {(void *)&g, (void *)&ctl, (void *)&acc, (void *)&tol, (void *)&max_iter, (void *)&m,
-                  spectral ? (void *)&so : (void *)&mg};
-  // precond 2: the spectral preconditioner where the transform covers the grid; multigrid elsewhere and for precond 1
+  so.limit = spectral ? spectral_limit(c, nb) : 0;
+  void *args[] = {(void *)&g, (void *)&ctl, (void *)&acc, (void *)&tol, (void *)&max_iter, (void *)&m, (void *)&mg,
+                  (void *)&c.mg_wh, (void *)&c.mg_wv, (void *)&so};  // (the last three: spectral only)
+  // precond 2: the spectral preconditioner where the transform covers the grid, while it is the faster one; multigrid
+  // elsewhere and for precond 1
   const void *fn = spectral ? (const void *)k_cg_loop_spectral
                             : (c.opt.precond != 0 ? (const void *)k_cg_loop<1, WEIGHTED>
                                                   : (const void *)k_cg_loop<0, WEIGHTED>);
@@ -1001,7 +1070,7 @@ cudaError_t solve_depth_async(Ctx &c) {
   for (int it = 0; it < c.opt.irls_iters; ++it) {
     k_irls_weights<<<nb, kThreads, 0, c.stream>>>(g, c.mg_wh, c.mg_wv, (double)c.opt.irls_delta);
     c.stats.launches += 1;
-    if (!direct_solve(c)) {  // the spectral preconditioner needs no hierarchy
+    if (!direct_solve(c)) {  // (a spectral solve builds the hierarchy if it goes over to it)
       for (int l = 0; l + 1 < mg.levels; ++l) {
         const int n = mg.H[l + 1] * mg.W[l + 1];
         k_mg_coarsen<<<(n + kThreads - 1) / kThreads, kThreads, 0, c.stream>>>(mg, l, c.mg_wh, c.mg_wv);
@@ -1110,10 +1179,16 @@ template <bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads, IRTPS_CG_BATCH_MINB) k_cg_loop_b(const CGJob *jobs, int n) {
   for_team<WEIGHTED>(jobs, n, [](const CGJob &j, Team t) {
     if (!WEIGHTED && j.direct) return;  // solved by the transform
-    if (WEIGHTED && j.direct)
-      cg_loop_body<2, true>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, &j.spec, t);
-    else if (j.pre == 1)
-      cg_loop_body<1, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, nullptr, t);
+    Progress p;
+    if (WEIGHTED && j.direct) {
+      if (j.spec.limit > 0) {
+        p = cg_loop_body<2, true>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, &j.spec, t);
+        if (!p.change) return;
+      }
+      mg_coarsen_all(j.mg, j.wh, j.wv, j.ctl, t);
+    }
+    if (j.pre == 1)
+      cg_loop_body<1, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, nullptr, t, p);
     else
       cg_loop_body<0, WEIGHTED>(j.g, j.ctl, &j.ds->cg, j.tol, j.max_iter, j.check, j.mg, nullptr, t);
   });
@@ -1189,7 +1264,10 @@ void cg_fill_job(Ctx &c, int nblk, int blk_begin, DevStats *ds, void *dst) {
   j.check = c.opt.cg_check_every > 0 ? c.opt.cg_check_every : 10;
   j.pre = c.opt.precond != 0 ? 1 : 0;  // iterative solves: multigrid for precond 1 and 2
   j.direct = direct_solve(c) ? 1 : 0;
-  if (j.direct) j.spec = spec_object(c, &ds->cg);
+  if (j.direct) {
+    j.spec = spec_object(c, &ds->cg);
+    j.spec.limit = spectral_limit(c, nblk);
+  }
   j.blk_begin = blk_begin;
   j.wh = c.mg_wh;
   j.wv = c.mg_wv;

@@ -380,6 +380,30 @@ SpecObj spec_object(const Ctx &c, CGAcc *acc) {
 
 size_t spec_line_smem(const Ctx &c) { return line_smem(c.sp.row, c.sp.col); }
 
+// Iterations after which a weighted solve on nblk blocks has taken as long with the spectral preconditioner as with the
+// multigrid one from the start, from the measured times of an iteration (us):
+//  - spectral: 12 for the barriers, and per line pair and block 2 + m / 100 a transform of m points (rows
+//    twice, columns both ways): 27 at 128 x 128, 49 at 375 x 421, 90 at 1024 x 1024, 332 at 2048 x 2048, 45 at 24 x 24 and
+//    150 at 2 x 1000, where the few blocks have many short lines each;
+//  - multigrid: 60 up to 4096 points (one block), else 90 + 11 for every point a thread: 100 at 128 x 128, 240 at
+//    1024 x 1024, 600 at 2048 x 2048; its iterations grow like 10 P^0.2 (50 at 64 x 64, 110 at 375 x 421, 210 at 2048 x
+//    2048 with 5 % outliers and a threshold of 1e-3).
+// So the limit is 54 at 24 x 24, 110 at 64 x 64, about 300 from 128 x 128 to 512 x 512, 390 at 2048 x 2048; below 24
+// (17 at 2 x 1000) multigrid does the whole solve, which on such strips takes 20 iterations whatever the weights.
+// Two reweightings with 5 % outliers at thresholds of 0.05, 1e-3 and 1e-4, ms: multigrid alone 17.1, 26.6, 30.1 at 256 x
+// 200 and 27.7, 41.1, 47.0 at 375 x 421; spectral alone 5.3, 28.4, 72.7 and 9.0, 47.8, 121; with the limit 5.4, 21.4,
+// 26.7 and 9.0, 29.6, 39.4.
+int spectral_limit(const Ctx &c, int nblk) {
+  const SpecObj &o = c.sp;
+  auto rounds = [&](int lines) { return (double)((lines + nblk - 1) / nblk); };
+  const double P = (double)c.H * c.W;
+  const double spectral = 12.0 + 2.0 * rounds(o.row_blocks) * (2.0 + 0.01 * o.row.m) +
+                          rounds((c.W + 1) / 2) * (2.0 + 0.02 * o.col.m);
+  const double multigrid = P <= 4096.0 ? 60.0 : 90.0 + 11.0 * P / (256.0 * nblk);
+  const int limit = (int)(10.0 * std::pow(P, 0.2) * multigrid / spectral);
+  return limit < 24 ? 0 : limit;
+}
+
 cudaError_t launch_spectral(Ctx &c) {
   const SpecObj o = spec_object(c, &c.dstats->cg);
   const size_t rs = row_smem(o), cs = col_smem(o);
