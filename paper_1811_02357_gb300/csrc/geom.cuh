@@ -390,11 +390,8 @@ __device__ __forceinline__ bool walker_finish_walk(Walker &m, const Field &f, F3
 #ifndef IRTPS_CLIMB
 #define IRTPS_CLIMB 2
 #endif
-#ifndef IRTPS_START_LEVEL
-#define IRTPS_START_LEVEL 3
-#endif
 constexpr int kClimb = IRTPS_CLIMB;
-constexpr int kStartLevel = IRTPS_START_LEVEL;  // level of a primary ray's march after a quick start
+constexpr int kStartLevel = 3;  // level of a primary ray's march after a quick start
 __device__ __forceinline__ void walker_cross(Walker &m, float tx, float ty, int top) {
   const int nx = m.nx + (tx <= ty ? 1 : 0), ny = m.ny + (ty <= tx ? 1 : 0);
   m.te = fminf(tx, ty);

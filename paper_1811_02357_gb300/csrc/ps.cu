@@ -503,10 +503,7 @@ struct PSList {
 #endif
 // resident blocks per SM asked of the normal-equation form (its state fits 64 registers at V <= 2)
 constexpr int kPsMinBlocks = IRTPS_PS_MINB;
-#ifndef IRTPS_PS_MINB1
-#define IRTPS_PS_MINB1 5
-#endif
-constexpr int kPsMinBlocks1 = IRTPS_PS_MINB1;  // one pixel a thread needs fewer registers
+constexpr int kPsMinBlocks1 = 5;  // one pixel a thread needs fewer registers
 // lights per unrolled step of the streaming loop, over all V pixels of a thread
 constexpr int kPsKUnroll = IRTPS_PS_KUNROLL;
 
@@ -599,10 +596,7 @@ __global__ void __launch_bounds__(256, (NE && V < 4) ? (V == 1 ? kPsMinBlocks1 :
 
 // The listed pixels, one per thread (the FP64 pipe is narrow: a pixel's FP64 work stays in
 // one lane), a grid-stride loop over the list.
-#ifndef IRTPS_PS_MASKED_BLOCKS
-#define IRTPS_PS_MASKED_BLOCKS 8
-#endif
-constexpr int kPsMaskedBlocks = IRTPS_PS_MASKED_BLOCKS;  // resident blocks per SM (its loads' latency bounds it)
+constexpr int kPsMaskedBlocks = 8;  // resident blocks per SM (its loads' latency bounds it)
 template <int C, typename TI>
 __global__ void __launch_bounds__(128, kPsMaskedBlocks) k_ps_masked(const PSArgs a, const PSList L) {
   const unsigned n = *L.count;

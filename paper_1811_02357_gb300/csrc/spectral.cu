@@ -56,10 +56,7 @@ __device__ __forceinline__ void spec_pass(const SpecObj &o, int blk) {
   if (PASS == SP_BACK) rows_back<DST_ADD>(o, blk);
   if (PASS == SP_BACK_LAST) rows_back<DST_ADD_LAST>(o, blk);
 }
-#ifndef IRTPS_COL_THREADS
-#define IRTPS_COL_THREADS 512
-#endif
-constexpr int kColThreads = IRTPS_COL_THREADS;  // threads of a column block
+constexpr int kColThreads = 512;  // threads of a column block
 template <int PASS>
 __global__ void __launch_bounds__(PASS == SP_COLS ? kColThreads : kSpecThreads) k_spec(const __grid_constant__ SpecObj o) {
   spec_pass<PASS>(o, blockIdx.x);

@@ -364,8 +364,10 @@ cudaError_t launch_horizon_batch(cudaStream_t s, const PyrObj *d_objs, int n, in
 // Environment: bilinear lookup in a C x EH x EW latitude-longitude map over the
 // full sphere (theta = acos(w_z) down the rows, phi = atan2(w_y, w_x) across,
 // texel centres at half-integers, wrap in phi, clamp in theta), every fused
-// multiply-add written out, so that a lookup's bits do not depend on the code around it.  Three
-// channels are stored as float4 texels: 4 loads a lookup instead of 12.
+// multiply-add written out, so that a lookup's bits do not depend on the code around it.  (One and three
+// channels fuse different products of a row's mix; both orders are kept as they were first compiled, since
+// a last-bit change of a lookup can send a later ray past an edge.)  Three channels are stored as float4
+// texels: 4 loads a lookup instead of 12.
 // ---------------------------------------------------------------------------
 template <int C>
 __device__ __forceinline__ void env_lookup(const float *__restrict__ env, int EH, int EW, F3 w, float *out) {
@@ -466,16 +468,9 @@ constexpr int kTraceThreads = 128;
 constexpr int kMarchKeep = IRTPS_MARCH_KEEP;
 // node steps of a lane between two looks at the warp's lanes (one copy of the step, a rolled loop): four take 6 % off
 // the single-object traces (512 x 512: 96.6 -> 90.6 ms), the batched one loses 3 %
-#ifndef IRTPS_NODE_STEPS
-#define IRTPS_NODE_STEPS 4
-#endif
-#ifndef IRTPS_REFILL_BATCH
-#define IRTPS_REFILL_BATCH 18
-#endif
+constexpr int kSingleNodeSteps = 4, kBatchNodeSteps = 1;
 // set up again before marching while at least this many lanes of the warp have no ray to march
-#ifndef IRTPS_REFILL
-#define IRTPS_REFILL 14
-#endif
+constexpr int kSingleRefill = 14, kBatchRefill = 18;
 // run leaf steps once kLeafBatch * (lanes waiting for one) >= lanes doing node steps
 constexpr int kLeafBatch = IRTPS_LEAF_BATCH;
 enum : int { PH_SETUP = 0, PH_MARCH = 1, PH_RESOLVE = 2, PH_DONE = 3, PH_LEAF = 4 };
@@ -726,7 +721,7 @@ __global__ void __launch_bounds__(kTraceThreads,
     if (live == 0u) break;
     // ---- march while enough of the live lanes are marching; node steps every
     // iteration, leaf steps once enough marching lanes wait for one ----
-    constexpr int kNodeSteps = BATCH ? 1 : IRTPS_NODE_STEPS, kRefill = BATCH ? IRTPS_REFILL_BATCH : IRTPS_REFILL;
+    constexpr int kNodeSteps = BATCH ? kBatchNodeSteps : kSingleNodeSteps, kRefill = BATCH ? kBatchRefill : kSingleRefill;
     const int n_live = __popc(live);
     int iters = 0;
     while (true) {
@@ -1031,16 +1026,12 @@ SharedSplit shared_split(int n_pix, int spp) {
 // stored and the sums are run afterwards (k_reduce_split), at most kSplitBytes of them (two passes over 256 MB take
 // 0.1 ms, the samples themselves ten times that).  Three iterations of a 64 x 64 object with 8
 // lights and 64 samples: 3.06 ms unsplit, 1.45 with 2^18 items, 1.31 with 2^19, 1.24 with 2^20.
-#ifndef IRTPS_SPLIT_ITEMS_LOG2
-#define IRTPS_SPLIT_ITEMS_LOG2 20
-#endif
-#ifndef IRTPS_SPLIT_MIN_CHUNK
-#define IRTPS_SPLIT_MIN_CHUNK 2
-#endif
+constexpr long long kSplitItems = 1ll << 20;
+constexpr int kSplitMinChunk = 2;
 SharedSplit light_split(const Ctx &c, int n_pix, int spp) {
   const long long items = (long long)n_pix * c.K;
-  long long n = (1ll << IRTPS_SPLIT_ITEMS_LOG2) / items;
-  const long long most = spp / IRTPS_SPLIT_MIN_CHUNK;
+  long long n = kSplitItems / items;
+  const long long most = spp / kSplitMinChunk;
   n = std::max(1ll, std::min(n, most));
   if (items * spp * c.C * 4 > kSplitBytes) n = 1;
   SharedSplit r;
