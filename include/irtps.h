@@ -288,17 +288,20 @@ int irtps_get_ps_tuning(irtps_ctx *ctx, int *pixels_per_thread); /* the width in
 int irtps_autotune(irtps_ctx *ctx, int spp_probe, int bounces, uint64_t seed, double *out_ms);
 
 /* ---- Batches: many objects, one launch per IRT stage ----
- * A batch runs the IRT loop of n_obj contexts together: per iteration one
- * batched pyramid launch per level, ONE persistent trace launch whose lanes take
+ * A batch runs the IRT loop of n_obj contexts together: per iteration two
+ * batched pyramid launches (one for small grids), ONE persistent trace launch whose lanes take
  * (object, light, pixel) work items from a shared queue (objects of larger
- * per-item cost first), one PS launch, one cooperative depth-solve launch in
- * which each object's solve runs on its own team of blocks, and one D_H launch.
+ * per-item cost first), one PS launch, the passes of the direct depth solves (one
+ * launch a pass, each object with its own number of refinements) and one
+ * cooperative launch of the iterative ones, in which each object's solve runs on
+ * its own team of blocks, and two small D_H launches.
  * Objects may differ in H, W, K, spp, bounces and options; all must have the
  * same C, image dtype, sampling option and irls_iters (robust integration runs
  * the same number of reweighting steps for every object; irls_delta may differ),
  * and none may have fill_holes (hole interpolation runs per context).  Every object's results are bit-identical to its own
- * irtps_iterate in the trace and the normal solve; the depth solve differs from
- * it only by the summation order of its reductions (team size), within cg_tol.
+ * irtps_iterate in the trace and the normal solve; so is a direct
+ * depth solve; an iterative one differs from it only by the summation order of its
+ * reductions (team size), within cg_tol.
  *
  * The batch keeps pointers to the caller's contexts, which must outlive it and
  * must not be used concurrently with a batch call.  irtps_batch_create sets the
@@ -313,7 +316,7 @@ int irtps_batch_set_stream(irtps_batch *b, void *stream);
  * x W_i, dtype IRTPS_F32 or IRTPS_F16, host pointers if on_device == 0, else
  * device pointers readable on the batch stream) into object i, then classic PS
  * (Eq. 4) and integration for all objects, as irtps_set_images does for one.
- * Results equal irtps_set_images' up to the summation order of the solve. */
+ * Results equal irtps_set_images' up to the summation order of iterative solves. */
 int irtps_batch_set_images(irtps_batch *b, const void *const *images, int dtype, int on_device);
 /* n_iter IRT iterations of every object (each context must have images set):
  * spp[i], bounces[i] for object i (host arrays of n_obj; bounces in 1..3); seed
