@@ -152,7 +152,7 @@ int irtps_set_stream(irtps_ctx *ctx, void *stream);
 int irtps_set_images(irtps_ctx *ctx, const void *images, int dtype, int on_device);
 
 /* IRT iterations (Sec. IV, stages 4-5 and the loop): n_iter times
- *   build the min/max pyramid of H_t; trace Lbar_t over (H_t, n_t, rho_t) with
+ *   build the pyramid of H_t; trace Lbar_t over (H_t, n_t, rho_t) with
  *   spp samples per (pixel, light) (per pixel with light-shared sampling) and
  *   bounces in 1..3 (the paper's r1..r3);
  *   I = A0 - rho_t * Lbar_t (subtracted from the ORIGINAL images); PS -> n, rho;
@@ -269,7 +269,7 @@ int irtps_set_object(irtps_ctx *ctx, uint32_t object);
  * plain walk reaches whatever the number of levels.
  *   blocks_per_sm : resident 128-thread blocks per SM of the persistent trace
  *                   grid (1 .. occupancy limit; 0 = the occupancy limit)
- *   mip_cut       : top levels of the min/max pyramid the march leaves out
+ *   mip_cut       : top levels of the pyramid the march leaves out
  *                   (0 = full depth; clamped so that two levels remain) */
 int irtps_set_tuning(irtps_ctx *ctx, int blocks_per_sm, int mip_cut);
 int irtps_get_tuning(irtps_ctx *ctx, int *blocks_per_sm, int *mip_cut);

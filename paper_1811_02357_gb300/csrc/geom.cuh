@@ -1,5 +1,5 @@
 // Device geometry of the reverted Monte-Carlo trace: random numbers, cosine
-// sampling, ray / triangle tests and the max-pyramid heightfield march.
+// sampling, ray / triangle tests and the heightfield march over a pyramid of bounding planes.
 //
 // Every operation whose result decides an integer (hit or miss, hit triangle,
 // hit pixel, shadow visibility) is written with explicitly rounded FP32

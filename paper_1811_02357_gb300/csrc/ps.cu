@@ -276,9 +276,9 @@ __device__ __forceinline__ void ps_rhs_twofold(const PSArgs &a, int p, unsigned 
 
 // Systems of a condition number up to kTwofoldCond are solved in FP32 and refined twice: G = M^-1 R from the FP32
 // inverse, then G += M^-1 (R - M G), the residual in twice the precision (M as hi + lo).  The error of the first G,
-// about 4 * 2^-24 cond relative (1.2e-4 at 512), is squared by the first step; the second one's correction is about
-// an ulp of G, known to 1e-4 of itself, so that G is the exact solution's rounding but for one pixel in ten
-// thousand or fewer.  Such a system is certainly below cond_max.  Beyond it the inverse and the products are FP64, whose 130 or so
+// a few times 2^-24 cond relative (3e-4 to 7e-4 at worst over thousands of clustered light sets with condition numbers to
+// 512, on the CPU), is squared by the first step, to a few ulp of G; the second one's correction is known to 7e-4 of
+// itself, so that G is the exact solution's rounding but for one pixel in a hundred or fewer, an ulp off.  Such a system is certainly below cond_max.  Beyond it the inverse and the products are FP64, whose 130 or so
 // operations a pixel bound this kernel (16 cycles of the SM's FP64 pipe per warp instruction).
 constexpr double kTwofoldCond = 512.0;
 
